@@ -263,7 +263,10 @@ int btdf_profile_read(btdf_ctx *ctx, double *ms_ib, double *ms_lbm, int64_t *lau
 #define BTDF_VARIANT_COUNT 14
 
 /* Variant of the fused collide-stream kernel.  Results do not depend on it.
- *   0 automatic: on lattices of at least 2^23 nodes 11 for FP32 and 12 for
+ *   0 automatic: two steps per pass over the lattice where the call's steps come
+ *     in pairs and that is the faster form (nf = 1, no box, every marker support
+ *     inside the lattice and off the inlet and outlet columns; FP32 storage with
+ *     bodies: from 2^17 nodes up); single steps otherwise: on lattices of at least 2^23 nodes 11 for FP32 and 12 for
  *     FP16 / BF16 storage (11 where no tensor maps could be encoded), on
  *     smaller ones 2 for FP32 and 11 for FP16 / BF16 (the autotuner's usual
  *     picks on a GB300)
@@ -320,7 +323,9 @@ int btdf_device_bytes(const btdf_ctx *ctx, size_t *bytes);
  * time (the mean of the middle half of the sorted times).  The
  * populations, the step counter, the force history and the last step's
  * marker results are restored afterwards, so the simulation does not
- * advance.  Outputs (may be NULL): *chosen, and ms[v] = that mean, in ms per step, of
+ * advance.  Where pairs of steps can run (btdf_tune, variant 0) they are timed
+ * too, ms[0] being half a pair's time; if that is the lowest, pairs stay on and
+ * the chosen variant takes the remaining single steps.  Outputs (may be NULL): *chosen, and ms[v] = that mean, in ms per step, of
  * variant v for v = 0..BTDF_VARIANT_COUNT-1 (-1 where not timed).  Needs temporary device memory
  * for one copy of the populations and, with flush_l2, four times the L2 size.
  * Synchronizes.  Errors: EINVAL (steps outside 1..100000), ESTATE (no fields),

@@ -98,8 +98,14 @@ def tune_lattice(lat, cache: Optional[TuneCache] = None, steps: int = 20, flush_
     cache miss.  Returns the cache entry with ``cached`` set."""
     cache = cache or TuneCache()
     key = lattice_key(lat, device or device_name())
-    return _tune(lat, key, cache, lambda: lat.autotune(steps, flush_l2), lambda v: lat.tune(v, 0),
-                 retune)
+    entry = _tune(lat, key, cache, lambda: lat.autotune(steps, flush_l2), lambda v: lat.tune(v, 0),
+                  retune)
+    if not entry["cached"]:
+        entry = dict(entry, pairs=bool(getattr(lat, "tuned_pairs", False)))
+        cache.put(key, {k: v for k, v in entry.items() if k != "cached"})
+    elif entry.get("pairs"):
+        lat.tune(0, 0)   # automatic: two steps per pass where they win
+    return entry
 
 
 def tune_batch(bt, cache: Optional[TuneCache] = None, steps: int = 10, flush_l2: bool = False,

@@ -211,6 +211,7 @@ class Lattice:
             raise BtdfError(rc, f"btdf_create: {btdf_status_string(rc)}")
         self._ctx = ctx
         self.body_markers = []
+        self.tuned_pairs = False      # autotune() found two steps per pass faster
 
     @classmethod
     def from_case(cls, case, storage=BTDF_F32, stream: int = 0, history_len=4096, drs=None,
@@ -363,6 +364,7 @@ class Lattice:
         ms = np.zeros(VARIANT_COUNT, dtype=np.float32)
         self._check(lib().btdf_autotune(self._ctx, int(steps), 1 if flush_l2 else 0, C.byref(ch),
                                         ms.ctypes.data), "btdf_autotune")
+        self.tuned_pairs = 0 < ms[0] < min(ms[v] for v in range(1, VARIANT_COUNT) if ms[v] >= 0)
         return ch.value, {v: float(ms[v]) for v in range(1, VARIANT_COUNT) if ms[v] >= 0}
 
     def set_wait_limit(self, polls):

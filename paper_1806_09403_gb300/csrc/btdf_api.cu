@@ -83,6 +83,7 @@ namespace {
 
 constexpr int kGraphSteps = 64;          // steps per replayed CUDA graph (even)
 constexpr int kFullGrid = 1 << 30;       // grid cap meaning "one row segment per warp"
+constexpr int kSchedWords = 3;           // device counters: the two of LatticeParams.sched, pair_kernel's
 constexpr int kStageSlots = 4;           // pinned staging slots for marker velocities
 constexpr uint64_t kStateMagic = 0x3230465444544242ull;   // "BBTDTF02"
 
@@ -175,13 +176,25 @@ struct btdf_ctx {
     int* d_seg_index = nullptr;
     int* d_seg_ptr = nullptr;
     CsrEntry* d_csr = nullptr;
+    // Pairs of steps (PairForces): the band rows of the strip pairs, their nodes
+    // with spread terms, and the spread forces of either step.
+    // Built for the first pair after the markers change, in one allocation.
+    void* d_pair = nullptr;
+    size_t pair_bytes = 0;
+    int* d_strip_row = nullptr;
+    int4* d_bnodes = nullptr;
+    float* d_fb[2] = {nullptr, nullptr};
+    int nbnode = 0;
     int* d_body_ptr = nullptr;
     double* d_body_scale = nullptr;
     double2* d_hist = nullptr;
     unsigned long long* d_step = nullptr;
     int* d_status = nullptr;
     unsigned* d_sched = nullptr;         // tile tickets of the warp-specialized TMA kernel
-    float* d_outlet = nullptr;         // [9][ny] previous outlet column (convective outlet)
+    // [9][ny] outlet column of the last step (convective outlet): d_outlet[b]
+    // belongs to population buffer b
+    float* d_outlet[2] = {nullptr, nullptr};
+    int sms = 1;
     float2* d_box = nullptr;           // perimeter velocities of the prescribed-velocity box
     std::vector<MarkerAux> aux_host;
     // Pinned host staging, so per-step host <-> device copies are true DMA
@@ -196,11 +209,15 @@ struct btdf_ctx {
     void* pin = nullptr;               // force-history read-back
     size_t pin_cap = 0;
 
+    // Every marker support lies inside the lattice, off the inlet and outlet
+    // columns (set by rebuild_markers): ib_pair_kernel's condition.
+    bool markers_inside = true;
     cudaGraphExec_t gexec[2] = {nullptr, nullptr};
     long long pf_grid[2] = {1, 1};                 // software-pipelined kernel [npl 4/2]
     long long pf_units[2][2] = {};                 // L2 prefetch distance of variants 10, 11 [local/pull]
     long long tma_grid[kVarCount] = {};  // persistent grid of each TMA variant
     int variant = kVarAuto;              // LBM kernel variant (btdf_tune)
+    bool pairs_tuned = false;            // the autotuner found pairs of steps faster than `variant`
     int grid_override = 0;               // 0: SMs x resident blocks
     bool tma_ok = false;                 // tensor maps encoded
     CUtensorMap tmap[2][3];              // [buffer][box of 10 / 18 / 9 rows]
@@ -217,6 +234,7 @@ struct btdf_ctx {
     // creation-time inflow speed; btdf_set_inflow changes only cfg.u_in.
     double u_ref = 0.0;
     std::vector<int> band_keys;        // y * nseg + segment of each band segment
+    std::vector<int> seg_ptr_host;     // the spreading table's row pointers
     long long marker_gen = 0;          // bumped by every rebuild of the marker tables
     AdjointTape tape;
     double2* tune_hist = nullptr;      // one-slot force ring used while btdf_autotune times steps
@@ -273,6 +291,9 @@ void free_markers(btdf_ctx* ctx) {
     ctx->dev_bytes -= ctx->marker_bytes;
     ctx->marker_bytes = 0;
     dfree(ctx, ctx->d_arena);
+    ctx->dev_bytes -= ctx->pair_bytes;
+    ctx->pair_bytes = 0;
+    dfree(ctx, ctx->d_pair);
     ctx->d_mk = nullptr;
     ctx->d_aux = nullptr;
     ctx->d_F[0] = ctx->d_F[1] = nullptr;
@@ -281,6 +302,10 @@ void free_markers(btdf_ctx* ctx) {
     ctx->d_seg_index = nullptr;
     ctx->d_seg_ptr = nullptr;
     ctx->d_csr = nullptr;
+    ctx->d_fb[0] = ctx->d_fb[1] = nullptr;
+    ctx->d_bnodes = nullptr;
+    ctx->d_strip_row = nullptr;
+    ctx->nbnode = 0;
     ctx->d_body_ptr = nullptr;
     ctx->d_body_scale = nullptr;
     ctx->d_hist = nullptr;
@@ -342,7 +367,8 @@ int auto_variant(const btdf_ctx* ctx) {
 // Tensor map of a TMA variant: boxes of 10, 18 and 9 rows.
 int tmap_index(int v) { return v == kVarTma16x2 ? 1 : v == kVarTmaWs7x3 ? 2 : 0; }
 
-LatticeParams lattice_params(const btdf_ctx* ctx) {
+// Description of the lattice for kernels that read buffer `cur`.
+LatticeParams lattice_params(const btdf_ctx* ctx, int cur) {
     LatticeParams p{};
     p.nx = ctx->cfg.nx;
     p.ny = ctx->cfg.ny;
@@ -355,7 +381,8 @@ LatticeParams lattice_params(const btdf_ctx* ctx) {
     p.bcx = box ? kBcxPeriodic : ctx->cfg.bc_x == BTDF_BCX_CONVECTIVE ? kBcxInout : ctx->cfg.bc_x;
     p.bcy = box ? kBcyPeriodic : ctx->cfg.bc_y;
     p.box = ctx->d_box;
-    p.outlet = ctx->d_outlet;
+    p.outlet = ctx->d_outlet[cur];
+    p.outlet_out = ctx->d_outlet[1 - cur];
     p.uc_old = (float)(1.0 / (1.0 + ctx->cfg.u_in));
     p.uc_new = (float)(ctx->cfg.u_in / (1.0 + ctx->cfg.u_in));
     p.omega = (float)(1.0 / ctx->cfg.tau);
@@ -420,7 +447,7 @@ cudaEvent_t next_event(btdf_ctx* ctx) {
 
 // Issues the kernels of one time step reading buffer `cur` (Algorithm 1).
 int enqueue_step(btdf_ctx* ctx, cudaStream_t st, bool pull, int cur, bool prof) {
-    const LatticeParams p = lattice_params(ctx);
+    const LatticeParams p = lattice_params(ctx, cur);
     cudaEvent_t e0 = nullptr, e1 = nullptr, e2 = nullptr;
     if (prof) {
         e0 = next_event(ctx);
@@ -480,14 +507,126 @@ int enqueue_step(btdf_ctx* ctx, cudaStream_t st, bool pull, int cur, bool prof) 
     return BTDF_OK;
 }
 
+// Whether pairs of steps (btdf_pair.cu) can run: no box, single-pass forcing and
+// supports that ib_pair_kernel covers.
+bool pairs_possible(const btdf_ctx* ctx) {
+    return !ctx->prof && !ctx->d_box && (ctx->nmark == 0 || (ctx->cfg.nf == 1 && ctx->markers_inside));
+}
+
+// Whether the context takes them: with the automatic variant where they are the
+// faster form, or after the autotuner found them so.  With bodies a pair's chain
+// of four launches takes about 12 us; two single steps of a small FP32 lattice
+// take as long (160 x 80: 12.2 against 12.7 us; 800 x 400: 14.5 against 14.3;
+// 1200 x 600: 19.0 against 15.2), the slower 16-bit steps do not (160 x 80: 17.4
+// against 12.7).  Without bodies there is no chain (160 x 80: 7.6 against 4.0).
+bool pairs_allowed(const btdf_ctx* ctx) {
+    if (!pairs_possible(ctx)) return false;
+    if (ctx->variant != kVarAuto || ctx->grid_override != 0) return ctx->pairs_tuned;
+    return ctx->nmark == 0 || ctx->cfg.storage != kStoreF32 || (long long)ctx->cfg.nx * ctx->cfg.ny >= (1ll << 17);
+}
+
+// Tables of the pair kernels for the current markers.
+int ensure_pair_tables(btdf_ctx* ctx) {
+    if (ctx->nmark == 0 || ctx->d_pair) return BTDF_OK;
+    const int nx = ctx->cfg.nx, ny = ctx->cfg.ny;
+    const bool px = ctx->cfg.bc_x == kBcxPeriodic;
+    const std::vector<int>& seg_ptr = ctx->seg_ptr_host;
+    // the band as the pair kernel's strips see it, with the columns beside them:
+    // a node near a border belongs to two strips (and, wrapped, a narrow
+    // periodic lattice's node to several)
+    const LatticeParams lp = lattice_params(ctx, ctx->cur);
+    const int npl = pair_npl(ctx->cfg.storage, lp.bcx, nx, ny);
+    const int nstrip = pair_strips(lp, npl), own = pair_own(npl);
+    std::vector<int> strip_row((size_t)ny * nstrip, -1);
+    std::vector<int4> bnodes;
+    int nsrow = 0;
+    for (int s = 0; s < ctx->nband; s++)
+        for (int i = 0; i < kSeg; i++) {
+            const int b = seg_ptr[(size_t)s * (kSeg + 1) + i], e = seg_ptr[(size_t)s * (kSeg + 1) + i + 1];
+            if (e <= b) continue;
+            const int y = ctx->band_keys[s] / ctx->nseg, xn = ctx->band_keys[s] % ctx->nseg * kSeg + i;
+            for (int x = px ? xn - nx : xn; x < nstrip * own + npl; x += nx) {
+                for (int k = std::max(0, (x - npl) / own); k < nstrip; k++) {
+                    const int c = x - (k * own - npl);
+                    if (c < 0) break;
+                    if (c >= 32 * npl) continue;
+                    int& row = strip_row[(size_t)y * nstrip + k];
+                    if (row < 0) row = nsrow++;
+                    bnodes.push_back(make_int4(row * 64 * npl + c, b, e, 0));
+                }
+                if (!px) break;
+            }
+        }
+    const size_t fb_bytes = sizeof(float) * 64 * npl * (size_t)std::max(nsrow, 1);
+    Arena A;
+    const size_t o_srow = A.take<int>(sizeof(int) * strip_row.size());
+    const size_t o_bn = A.take<int4>(sizeof(int4) * std::max<size_t>(bnodes.size(), 1));
+    const size_t o_fb0 = A.take<float>(fb_bytes);
+    const size_t o_fb1 = A.take<float>(fb_bytes);
+    const size_t before = ctx->dev_bytes;
+    const cudaError_t ea = dalloc(ctx, &ctx->d_pair, A.size);
+    if (ea != cudaSuccess)
+        return ea == cudaErrorMemoryAllocation ? fail(ctx, BTDF_ENOMEM, "pair tables do not fit")
+                                               : cuda_fail(ctx, ea, "cudaMalloc");
+    ctx->pair_bytes = ctx->dev_bytes - before;
+    char* base = (char*)ctx->d_pair;
+    ctx->d_strip_row = (int*)(base + o_srow);
+    ctx->d_bnodes = (int4*)(base + o_bn);
+    ctx->nbnode = (int)bnodes.size();
+    ctx->d_fb[0] = (float*)(base + o_fb0);
+    ctx->d_fb[1] = (float*)(base + o_fb1);
+    cudaStream_t st = ctx->stream;
+    CK(cudaMemcpyAsync(ctx->d_strip_row, strip_row.data(), sizeof(int) * strip_row.size(), cudaMemcpyHostToDevice, st));
+    if (!bnodes.empty())
+        CK(cudaMemcpyAsync(ctx->d_bnodes, bnodes.data(), sizeof(int4) * bnodes.size(), cudaMemcpyHostToDevice, st));
+    // band nodes without terms keep a zero force
+    for (float* fb : ctx->d_fb) CK(cudaMemsetAsync(fb, 0, fb_bytes, st));
+    CK(cudaStreamSynchronize(st));
+    return BTDF_OK;
+}
+
+// Issues the kernels of two pulling time steps reading buffer `cur`; the state
+// is then in the other buffer.
+int enqueue_pair(btdf_ctx* ctx, cudaStream_t st, int cur) {
+    const LatticeParams p = lattice_params(ctx, cur);
+    PairForces f{};
+    f.F1 = ctx->d_F[1];   // p.F = d_F[0]: the last step's forces
+    f.strip_row = ctx->nmark > 0 ? ctx->d_strip_row : nullptr;
+    f.nodes = ctx->d_bnodes;
+    f.nnode = ctx->nbnode;
+    f.npl = pair_npl(ctx->cfg.storage, p.bcx, p.nx, p.ny);
+    f.nstrip = pair_strips(p, f.npl);
+    for (int a = 0; a < 9; a++) f.kin[a] = p.poff[a] + (unsigned)(1 - ey(a)) * p.rs;
+    f.fb1 = ctx->d_fb[1];
+    f.fb2 = ctx->d_fb[0];
+    f.done = ctx->d_sched + 2;
+    if (ctx->nmark > 0) {
+        IbParams q{};
+        q.nmark = ctx->nmark;
+        q.mk = ctx->d_mk;
+        q.aux = ctx->d_aux;
+        q.F_out = ctx->d_F[1];
+        q.Us = ctx->d_Us;
+        q.rhol = ctx->d_rhol;
+        q.first_pass = 1;
+        q.status = ctx->d_status;
+        CK(launch_ib_force(ctx->cfg.storage, true, ctx->width, ctx->g[cur], p, q, true, st));
+        q.F_out = ctx->d_F[0];
+        CK(launch_ib_pair(ctx->cfg.storage, ctx->width, ctx->g[cur], p, q, f, true, st));
+    }
+    CK(launch_pair(ctx->cfg.storage, ctx->g[cur], ctx->g[1 - cur], p, f, ctx->nmark > 0, st));
+    return BTDF_OK;
+}
+
 int ensure_graph(btdf_ctx* ctx, int cur) {
     if (ctx->gexec[cur]) return BTDF_OK;
     cudaGraph_t graph = nullptr;
     CK(cudaStreamBeginCapture(ctx->cap, cudaStreamCaptureModeThreadLocal));
     int rc = BTDF_OK;
     int c = cur;
-    for (int i = 0; i < kGraphSteps && rc == BTDF_OK; i++) {
-        rc = enqueue_step(ctx, ctx->cap, true, c, false);
+    const int per = pairs_allowed(ctx) ? 2 : 1;
+    for (int i = 0; i < kGraphSteps && rc == BTDF_OK; i += per) {
+        rc = per == 2 ? enqueue_pair(ctx, ctx->cap, c) : enqueue_step(ctx, ctx->cap, true, c, false);
         c = 1 - c;
     }
     cudaError_t e = cudaStreamEndCapture(ctx->cap, &graph);
@@ -556,7 +695,6 @@ int rebuild_markers(btdf_ctx* ctx) {
     const int nx = ctx->cfg.nx, ny = ctx->cfg.ny;
     const bool px = ctx->cfg.bc_x == kBcxPeriodic, py = ctx->cfg.bc_y == kBcyPeriodic;
     const int nm = ctx->nmark, nb = (int)ctx->bodies.size();
-    (void)nx;
     if (nm == 0) return BTDF_OK;
     std::vector<BodyDesc> descs;
     std::vector<int> body_ptr(nb + 1);
@@ -577,9 +715,17 @@ int rebuild_markers(btdf_ctx* ctx) {
         Body& B = ctx->bodies[b];
         B.wsum.assign(t.wsum.begin() + B.first, t.wsum.begin() + B.first + B.n);
     }
+    ctx->markers_inside = true;
+    for (const Body& B : ctx->bodies)
+        for (int l = 0; l < B.n; l++) {
+            const int i0 = (int)std::floor(B.X[l] - 0.5 * ctx->width) + 1, i1 = i0 + ctx->width - 1;
+            const int j0 = (int)std::floor(B.Y[l] - 0.5 * ctx->width) + 1, j1 = j0 + ctx->width - 1;
+            if ((!px && (i0 < 1 || i1 > nx - 2)) || (!py && (j0 < 0 || j1 > ny - 1))) ctx->markers_inside = false;
+        }
     ctx->aux_host = t.aux;
     CK(cudaMallocHost((void**)&ctx->aux_pin, sizeof(MarkerAux) * nm * kStageSlots));
     ctx->nband = (int)t.seg_keys.size();
+    ctx->seg_ptr_host = t.seg_ptr;
     const std::vector<Marker>& mk = t.mk;
     const std::vector<int>& seg_index = t.seg_index;
     const std::vector<int>& seg_ptr = t.seg_ptr;
@@ -646,7 +792,7 @@ int rebuild_markers(btdf_ctx* ctx) {
 }
 
 // Bytes of the convective outlet's column buffer (0 for other boundaries).
-size_t outlet_bytes(const btdf_ctx* ctx) { return ctx->d_outlet ? sizeof(float) * 9 * ctx->cfg.ny : 0; }
+size_t outlet_bytes(const btdf_ctx* ctx) { return ctx->d_outlet[0] ? sizeof(float) * 9 * ctx->cfg.ny : 0; }
 
 // Marker positions must be finite and their support must touch the lattice.
 // Under the convective outlet no support may reach the outlet column: the IB
@@ -693,7 +839,7 @@ int tape_step(btdf_ctx* ctx, int64_t n, const float* gin, float* gout, cudaStrea
     AdjointTape& T = ctx->tape;
     const bool pull = tape_pull(T, n);
     float2* F = T.Fall + (size_t)n * ctx->nmark;
-    LatticeParams p = lattice_params(ctx);
+    LatticeParams p = lattice_params(ctx, ctx->cur);
     p.F = F;
     p.nbody = 0;
     p.step = nullptr;
@@ -765,7 +911,7 @@ int tape_backward_enqueue(btdf_ctx* ctx, cudaStream_t st) {
         const int rc = tape_run(ctx, j, s, e - 1, st);
         if (rc != BTDF_OK) return rc;
         for (int64_t n = e - 1; n >= s; n--) {
-            LatticeParams p = lattice_params(ctx);
+            LatticeParams p = lattice_params(ctx, ctx->cur);
             p.F = T.Fall + (size_t)n * nm;
             CK(cudaMemsetAsync(T.lam[1 - c], 0, sb, st));
             CK(launch_adjoint_step(tape_state(T, j, n), T.lam[c], T.lam[1 - c], p, q, ctx->width,
@@ -966,6 +1112,7 @@ int btdf_create(const btdf_config* cfg, void* stream, btdf_ctx** out) {
         if (cudaGetDevice(&dev) != cudaSuccess ||
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
             return bail(BTDF_ECUDA);
+        ctx->sms = sms;
         for (int v = 0; v < kVarCount; v++)
             if (is_tma(v)) ctx->tma_grid[v] = (long long)sms * collide_stream_tma_blocks_per_sm(c.storage, v);
         ctx->pf_grid[0] = (long long)sms * collide_stream_blocks_per_sm(c.storage, true, kVarReg4Pf);
@@ -995,15 +1142,16 @@ int btdf_create(const btdf_config* cfg, void* stream, btdf_ctx** out) {
     *ctx->status_pin = 0;
     if (dalloc(ctx, &ctx->d_step, sizeof(unsigned long long)) != cudaSuccess ||
         dalloc(ctx, &ctx->d_status, sizeof(int)) != cudaSuccess ||
-        dalloc(ctx, &ctx->d_sched, 2 * sizeof(unsigned)) != cudaSuccess ||
-        (c.bc_x == BTDF_BCX_CONVECTIVE && dalloc(ctx, &ctx->d_outlet, sizeof(float) * 9 * c.ny) != cudaSuccess) ||
+        dalloc(ctx, &ctx->d_sched, kSchedWords * sizeof(unsigned)) != cudaSuccess ||
+        (c.bc_x == BTDF_BCX_CONVECTIVE && (dalloc(ctx, &ctx->d_outlet[0], sizeof(float) * 9 * c.ny) != cudaSuccess ||
+                                            dalloc(ctx, &ctx->d_outlet[1], sizeof(float) * 9 * c.ny) != cudaSuccess)) ||
         (c.bc_x == BTDF_BCX_BOX && dalloc(ctx, &ctx->d_box, sizeof(float2) * (2 * c.nx + 2 * (c.ny - 2))) != cudaSuccess))
         return bail(BTDF_ECUDA);
     if (ctx->d_box && cudaMemsetAsync(ctx->d_box, 0, sizeof(float2) * (2 * c.nx + 2 * (c.ny - 2)), ctx->stream) != cudaSuccess)
         return bail(BTDF_ECUDA);
     if (cudaMemsetAsync(ctx->d_step, 0, sizeof(unsigned long long), ctx->stream) != cudaSuccess ||
         cudaMemsetAsync(ctx->d_status, 0, sizeof(int), ctx->stream) != cudaSuccess ||
-        cudaMemsetAsync(ctx->d_sched, 0, 2 * sizeof(unsigned), ctx->stream) != cudaSuccess ||
+        cudaMemsetAsync(ctx->d_sched, 0, kSchedWords * sizeof(unsigned), ctx->stream) != cudaSuccess ||
         cudaStreamSynchronize(ctx->stream) != cudaSuccess)
         return bail(BTDF_ECUDA);
     *out = ctx;
@@ -1021,7 +1169,8 @@ int btdf_destroy(btdf_ctx* ctx) {
     dfree(ctx, ctx->d_step);
     dfree(ctx, ctx->d_status);
     dfree(ctx, ctx->d_sched);
-    dfree(ctx, ctx->d_outlet);
+    dfree(ctx, ctx->d_outlet[0]);
+    dfree(ctx, ctx->d_outlet[1]);
     dfree(ctx, ctx->d_box);
     for (cudaEvent_t e : ctx->ev) cudaEventDestroy(e);
     for (cudaEvent_t e : ctx->aux_ev)
@@ -1050,12 +1199,13 @@ int btdf_init_fields(btdf_ctx* ctx, const double* rho, const double* ux, const d
         const size_t bytes = (size_t)9 * ctx->plane * ctx->elem;
         CK(cudaMemsetAsync(ctx->g[0], 0, bytes, st));
         CK(cudaMemsetAsync(ctx->g[1], 0, bytes, st));
-        if (ctx->d_outlet) CK(cudaMemsetAsync(ctx->d_outlet, 0, sizeof(float) * 9 * ctx->cfg.ny, st));
-        const LatticeParams p = lattice_params(ctx);
+        for (float* o : ctx->d_outlet)
+            if (o) CK(cudaMemsetAsync(o, 0, sizeof(float) * 9 * ctx->cfg.ny, st));
+        const LatticeParams p = lattice_params(ctx, ctx->cur);
         CK(launch_init_equilibrium(ctx->cfg.storage, ctx->g[0], p, d, d + nn, d + 2 * nn, st));
         CK(cudaMemsetAsync(ctx->d_step, 0, sizeof(unsigned long long), st));
         CK(cudaMemsetAsync(ctx->d_status, 0, sizeof(int), st));
-        CK(cudaMemsetAsync(ctx->d_sched, 0, 2 * sizeof(unsigned), st));
+        CK(cudaMemsetAsync(ctx->d_sched, 0, kSchedWords * sizeof(unsigned), st));
         CK(cudaStreamSynchronize(st));
         return BTDF_OK;
     };
@@ -1172,6 +1322,11 @@ int btdf_step(btdf_ctx* ctx, int64_t nsteps) {
     if (nsteps < 0) return fail(ctx, BTDF_EINVAL, "nsteps < 0");
     if (!ctx->has_fields) return fail(ctx, BTDF_ESTATE, "call btdf_init_fields or btdf_load_state first");
     int64_t i = 0;
+    const bool pairs = nsteps - (ctx->poststream ? 1 : 0) >= 2 && pairs_allowed(ctx);
+    if (pairs) {
+        const int rc = ensure_pair_tables(ctx);
+        if (rc != BTDF_OK) return rc;
+    }
     if (nsteps > 0 && ctx->poststream) {
         const int rc = enqueue_step(ctx, ctx->stream, false, ctx->cur, ctx->prof);
         if (rc != BTDF_OK) return rc;
@@ -1187,10 +1342,13 @@ int btdf_step(btdf_ctx* ctx, int64_t nsteps) {
             i += kGraphSteps;
         }
     }
-    for (; i < nsteps; i++) {
-        const int rc = enqueue_step(ctx, ctx->stream, true, ctx->cur, ctx->prof);
+    while (i < nsteps) {
+        const bool two = pairs && nsteps - i >= 2;
+        const int rc = two ? enqueue_pair(ctx, ctx->stream, ctx->cur)
+                           : enqueue_step(ctx, ctx->stream, true, ctx->cur, ctx->prof);
         if (rc != BTDF_OK) return rc;
         ctx->cur = 1 - ctx->cur;
+        i += two ? 2 : 1;
     }
     ctx->steps += nsteps;
     return BTDF_OK;
@@ -1272,7 +1430,7 @@ int btdf_read_field(btdf_ctx* ctx, int32_t kind, float* dst, int32_t dst_is_devi
     if (!dst_is_device) CK(cudaMalloc((void**)&d, sizeof(float) * nn));
     int rc = BTDF_OK;
     auto run = [&]() -> int {
-        const LatticeParams p = lattice_params(ctx);
+        const LatticeParams p = lattice_params(ctx, ctx->cur);
         if (kind >= 4) CK(launch_force_field(p, kind - 4, d, ctx->stream));
         else
             CK(launch_read_field(ctx->cfg.storage, !ctx->poststream, ctx->g[ctx->cur], p, kind, d,
@@ -1306,7 +1464,7 @@ int btdf_save_state(btdf_ctx* ctx, void* dst, size_t cap, size_t* used) {
     const size_t ob = outlet_bytes(ctx);
     CK(cudaMemcpyAsync((char*)dst + sizeof(h), ctx->g[ctx->cur], need - sizeof(h) - ob,
                        cudaMemcpyDeviceToHost, ctx->stream));
-    if (ob) CK(cudaMemcpyAsync((char*)dst + need - ob, ctx->d_outlet, ob, cudaMemcpyDeviceToHost, ctx->stream));
+    if (ob) CK(cudaMemcpyAsync((char*)dst + need - ob, ctx->d_outlet[ctx->cur], ob, cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
     if (used) *used = need;
     return read_status(ctx);
@@ -1328,7 +1486,7 @@ int btdf_load_state(btdf_ctx* ctx, const void* src, size_t len) {
     const size_t ob = outlet_bytes(ctx);
     CK(cudaMemcpyAsync(ctx->g[ctx->cur], (const char*)src + sizeof(h), need - sizeof(h) - ob,
                        cudaMemcpyHostToDevice, ctx->stream));
-    if (ob) CK(cudaMemcpyAsync(ctx->d_outlet, (const char*)src + need - ob, ob, cudaMemcpyHostToDevice, ctx->stream));
+    if (ob) CK(cudaMemcpyAsync(ctx->d_outlet[ctx->cur], (const char*)src + need - ob, ob, cudaMemcpyHostToDevice, ctx->stream));
     unsigned long long s = (unsigned long long)h.steps;
     CK(cudaMemcpyAsync(ctx->d_step, &s, sizeof(s), cudaMemcpyHostToDevice, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
@@ -1376,6 +1534,7 @@ int btdf_tune(btdf_ctx* ctx, int32_t variant, int32_t grid_blocks) {
     CK(cudaStreamSynchronize(ctx->stream));
     drop_graphs(ctx);
     ctx->variant = variant;
+    ctx->pairs_tuned = false;
     ctx->grid_override = grid_blocks;
     return BTDF_OK;
 }
@@ -1542,6 +1701,7 @@ int btdf_autotune(btdf_ctx* ctx, int32_t steps, int32_t flush_l2, int32_t* chose
     void* flush = nullptr;
     double2* th = nullptr;
     float2* fsave = nullptr;
+    float* osave = nullptr;
     const size_t nb = std::max<size_t>(ctx->bodies.size(), 1);
     std::vector<cudaEvent_t> ev;
     float res[kVarCount];
@@ -1554,6 +1714,10 @@ int btdf_autotune(btdf_ctx* ctx, int32_t steps, int32_t flush_l2, int32_t* chose
         if (flush_l2) CK(cudaMalloc(&flush, l2_flush_bytes()));
         CK(cudaMemcpyAsync(&counter0, ctx->d_step, sizeof(counter0), cudaMemcpyDeviceToHost, st));
         CK(cudaMemcpyAsync(save, ctx->g[cur0], pbytes, cudaMemcpyDeviceToDevice, st));
+        if (outlet_bytes(ctx)) {
+            CK(cudaMalloc((void**)&osave, outlet_bytes(ctx)));
+            CK(cudaMemcpyAsync(osave, ctx->d_outlet[cur0], outlet_bytes(ctx), cudaMemcpyDeviceToDevice, st));
+        }
         if (fbytes) {
             CK(cudaMemcpyAsync(fsave, ctx->d_F[0], fbytes, cudaMemcpyDeviceToDevice, st));
             CK(cudaMemcpyAsync(fsave + ctx->nmark, ctx->d_F[1], fbytes, cudaMemcpyDeviceToDevice, st));
@@ -1596,12 +1760,30 @@ int btdf_autotune(btdf_ctx* ctx, int32_t steps, int32_t flush_l2, int32_t* chose
                 best = v;
             }
         }
+        if (pairs_possible(ctx) && ctx->grid_override == 0) {   // pairs of steps, as time per step
+            const int rcp = ensure_pair_tables(ctx);
+            if (rcp != BTDF_OK) return rcp;
+            for (int i = 0; i < steps + 2; i++) {
+                if (flush) CK(launch_l2_flush(flush, l2_flush_bytes(), st));
+                const int e = std::max(i - 2, 0);
+                CK(cudaEventRecord(ev[2 * e], st));
+                int rc = enqueue_pair(ctx, st, ctx->cur);
+                if (rc != BTDF_OK) return rc;
+                CK(cudaEventRecord(ev[2 * e + 1], st));
+                ctx->cur = 1 - ctx->cur;
+            }
+            CK(cudaStreamSynchronize(st));
+            std::vector<float> t(steps);
+            for (int i = 0; i < steps; i++) CK(cudaEventElapsedTime(&t[i], ev[2 * i], ev[2 * i + 1]));
+            res[0] = 0.5f * interquartile_mean(t);
+        }
         return BTDF_OK;
     };
     int rc = run();
     // restore the state, the counter and the last step's marker results
     ctx->tune_hist = nullptr;
     ctx->variant = rc == BTDF_OK ? best : var0;
+    if (rc == BTDF_OK) ctx->pairs_tuned = res[0] > 0.0f && res[0] < res[best];
     ctx->cur = cur0;
     ctx->poststream = post0;
     ctx->steps = steps0;
@@ -1609,6 +1791,8 @@ int btdf_autotune(btdf_ctx* ctx, int32_t steps, int32_t flush_l2, int32_t* chose
     if (save) {
         e = cudaMemcpyAsync(ctx->g[cur0], save, pbytes, cudaMemcpyDeviceToDevice, st);
         if (e == cudaSuccess) e = cudaMemcpyAsync(ctx->d_step, &counter0, sizeof(counter0), cudaMemcpyHostToDevice, st);
+        if (e == cudaSuccess && osave)
+            e = cudaMemcpyAsync(ctx->d_outlet[cur0], osave, outlet_bytes(ctx), cudaMemcpyDeviceToDevice, st);
         if (e == cudaSuccess && fsave) {
             cudaMemcpyAsync(ctx->d_F[0], fsave, fbytes, cudaMemcpyDeviceToDevice, st);
             cudaMemcpyAsync(ctx->d_F[1], fsave + ctx->nmark, fbytes, cudaMemcpyDeviceToDevice, st);
@@ -1624,6 +1808,7 @@ int btdf_autotune(btdf_ctx* ctx, int32_t steps, int32_t flush_l2, int32_t* chose
     if (flush) cudaFree(flush);
     if (th) cudaFree(th);
     if (fsave) cudaFree(fsave);
+    if (osave) cudaFree(osave);
     drop_graphs(ctx);
     if (rc != BTDF_OK) return rc;
     if (e != cudaSuccess) return cuda_fail(ctx, e, "restoring the state after tuning");

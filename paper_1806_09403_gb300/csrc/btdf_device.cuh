@@ -273,7 +273,8 @@ __device__ __forceinline__ void y_source(int a, int y, const LatticeParams& p, i
             sy = y;
             pa = opposite(a);
             dx = 0;
-            add = -6.0f * wt(a) * (ex(a) * p.urx + ey(a) * p.ury);
+            // rounded by itself, so that no caller contracts it into its sum
+            add = __fmul_rn(-6.0f * wt(a), ex(a) * p.urx + ey(a) * p.ury);
         }
     }
 }
@@ -316,6 +317,18 @@ __device__ __noinline__ void pull_box_node(const T* __restrict__ g, const Lattic
                             eq_part_diff(a, p.urx, p.ury, m.dux, m.duy));
 }
 
+// Inlet node by non-equilibrium extrapolation from column 1, whose
+// post-streaming deviations are f1, to u = (u_in, 0).
+__device__ __forceinline__ void inlet_from(const float f1[9], const LatticeParams& p, float f[9]) {
+    const Moments m = moments(f1, p.urx, p.ury);
+    const float inx = p.u_in - p.urx, iny = -p.ury;
+#pragma unroll
+    for (int a = 0; a < 9; a++)
+        f[a] = f1[a] + wt(a) * m.rho *
+                           (eq_part_diff(a, p.urx, p.ury, inx, iny) -
+                            eq_part_diff(a, p.urx, p.ury, m.dux, m.duy));
+}
+
 // Post-streaming deviations with the boundary rules of the x ends: inlet
 // column by non-equilibrium extrapolation from column 1 to u = (u_in, 0),
 // f(0) = f(1) + f_eq(rho_1, u_in) - f_eq(rho_1, u*_1); outlet column copied
@@ -327,13 +340,7 @@ __device__ void pull_node(const T* __restrict__ g, const LatticeParams& p, int x
     if (p.bcx == kBcxInout && x == 0) {
         float f1[9];
         pull_raw<T>(g, p, 1, y, f1);
-        const Moments m = moments(f1, p.urx, p.ury);
-        const float inx = p.u_in - p.urx, iny = -p.ury;
-#pragma unroll
-        for (int a = 0; a < 9; a++)
-            f[a] = f1[a] + wt(a) * m.rho *
-                               (eq_part_diff(a, p.urx, p.ury, inx, iny) -
-                                eq_part_diff(a, p.urx, p.ury, m.dux, m.duy));
+        inlet_from(f1, p, f);
     } else if (p.bcx == kBcxInout && x == p.nx - 1) {
         pull_raw<T>(g, p, p.nx - 2, y, f);
         if (p.outlet != nullptr) {

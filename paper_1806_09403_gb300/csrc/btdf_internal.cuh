@@ -132,9 +132,11 @@ struct LatticeParams {
     float2 omop;
     float gx, gy;              // uniform body force
     // Convective outlet (null: zero-gradient): the outlet column's
-    // post-streaming deviations of the previous step, [9][ny], and the
-    // weights of f(N, t+1) = old / (1 + U) + U / (1 + U) f(N-1, t+1).
-    float* outlet;
+    // post-streaming deviations of the previous step, [9][ny], where this
+    // step's go, and the weights of
+    // f(N, t+1) = old / (1 + U) + U / (1 + U) f(N-1, t+1).
+    const float* outlet;
+    float* outlet_out;
     float uc_old, uc_new;
     // Prescribed-velocity box (null: none): every outer node gets the
     // velocity box[perimeter_index(x, y)] by non-equilibrium extrapolation
@@ -223,6 +225,36 @@ enum : int {
     kVarTmaWs7x3 = 13, // TMA tiles of 7 rows, a producer warp, 3 stages, <= 80 registers
     kVarCount = 14
 };
+// Columns a warp of the pair kernel owns with npl nodes per lane: those of its
+// lanes but the outer two.
+__host__ __device__ constexpr int pair_own(int npl) { return 30 * npl; }
+
+// What a pair of steps (btdf_pair.cu) needs besides LatticeParams.
+struct PairForces {
+    const float2* F1;          // Lagrangian forces of the first step (p.F: the second's)
+    // Spread over the band (Eq. 15): strip_row[y * nstrip + s] is the index of row
+    // y of strip s among the rows of strips that have terms, or -1 (null: no
+    // bodies); a row has the x, then the y components on the strip's 32 * npl
+    // columns; nodes[t] = (slot of the x component, first term, end of terms).
+    const int* strip_row;
+    const int4* nodes;
+    int nnode;
+    float *fb1, *fb2;          // spread forces of either step
+    unsigned* done;            // finished reduction blocks of pair_kernel, zero between launches
+    int nstrip, npl;           // strips, nodes per lane
+    unsigned kin[9];           // element offset of population a's source row from the row before
+};
+// Nodes per lane of the pair kernel for a lattice, and its strips.
+int pair_npl(int storage, int bcx, int nx, int ny);
+int pair_strips(const LatticeParams& p, int npl);
+
+// Two pulling steps in one kernel.
+cudaError_t launch_pair(int storage, const void* gin, void* gout, const LatticeParams& p, const PairForces& q,
+                        bool pdl, cudaStream_t st);
+// Marker forces of the second step of a pair from the state g before the first
+// and the first step's forces r.F1 (into q.F_out = p.F), and both steps' spread.
+cudaError_t launch_ib_pair(int storage, int width, const void* g, const LatticeParams& p, const IbParams& q,
+                           const PairForces& r, bool pdl, cudaStream_t st);
 // map: 3-D tensor map (x, y, population) of the input buffer with box
 // (128 + 2 * tma_halo(storage), tma_box_rows(variant), 9).
 cudaError_t launch_collide_stream_tma(int storage, int variant, const CUtensorMap* map, const void* gin,
