@@ -325,8 +325,9 @@ int btdf_device_bytes(const btdf_ctx *ctx, size_t *bytes);
  * marker results are restored afterwards, so the simulation does not
  * advance.  Where pairs of steps can run (btdf_tune, variant 0) they are timed
  * too, ms[0] being half a pair's time; if that is the lowest, pairs stay on and
- * the chosen variant takes the remaining single steps.  Outputs (may be NULL): *chosen, and ms[v] = that mean, in ms per step, of
- * variant v for v = 0..BTDF_VARIANT_COUNT-1 (-1 where not timed).  Needs temporary device memory
+ * the chosen variant takes the remaining single steps.  Outputs (may be NULL):
+ * *chosen, and ms[v] = that mean, in ms per step, of variant v for
+ * v = 0..BTDF_VARIANT_COUNT-1 (-1 where not timed).  Needs temporary device memory
  * for one copy of the populations and, with flush_l2, four times the L2 size.
  * Synchronizes.  Errors: EINVAL (steps outside 1..100000), ESTATE (no fields),
  * ENOMEM / ECUDA. */
@@ -355,9 +356,9 @@ int btdf_autotune(btdf_ctx *ctx, int32_t steps, int32_t flush_l2, int32_t *chose
  * Errors: EINVAL, ESTATE (no fields or no bodies), ENOMEM, EUNSTABLE.
  *
  * btdf_adjoint_backward reverses the last forward window: segments are
- * recomputed from their checkpoints, then each step is reversed by three
- * kernels (collision and boundary folds, marker forces and positions,
- * interpolation at the band nodes).  Outputs (host, any may be NULL):
+ * recomputed from their checkpoints, then each step is reversed by two
+ * kernels (marker forces and positions; collision, interpolation and boundary
+ * folds).  Outputs (host, any may be NULL):
  * dJdU = dJ/du_in, dJdX[l], dJdY[l] = dJ/dX_l, dJ/dY_l for every marker in the
  * order the markers were added.  Setting the inflow, moving markers or
  * changing marker velocities invalidates the window (ESTATE).  Synchronizes.

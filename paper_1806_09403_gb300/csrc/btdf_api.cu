@@ -131,9 +131,6 @@ struct AdjointTape {
     AdjMarker* am = nullptr;
     float* cscale = nullptr;
     float2* objw = nullptr;
-    int* band_keys = nullptr;
-    float* fbar_band = nullptr;
-    float2* Fbar_band = nullptr;
     float4* mbar = nullptr;
     double* acc = nullptr;       // [2 nmark + 1]: dJ/dX, dJ/dY, inlet part of dJ/dU
     size_t bytes = 0;
@@ -144,7 +141,7 @@ struct AdjointTape {
     std::vector<double> fwd_key, bwd_key;
     int cap_ck = 0, cap_every = 0;
     int64_t cap_F = 0;
-    int cap_mark = 0, cap_band = 0;
+    int cap_mark = 0;
 };
 
 }  // namespace
@@ -337,9 +334,6 @@ void free_tape(btdf_ctx* ctx) {
     dfree(ctx, T.am);
     dfree(ctx, T.cscale);
     dfree(ctx, T.objw);
-    dfree(ctx, T.band_keys);
-    dfree(ctx, T.fbar_band);
-    dfree(ctx, T.Fbar_band);
     dfree(ctx, T.mbar);
     dfree(ctx, T.acc);
     ctx->dev_bytes -= T.bytes;
@@ -854,8 +848,8 @@ int tape_step(btdf_ctx* ctx, int64_t n, const float* gin, float* gout, cudaStrea
     q.rhol = T.rhol;
     q.first_pass = 1;
     q.status = ctx->d_status;
-    CK(launch_ib_force(kStoreF32, pull, ctx->width, gin, p, q, false, st));
-    CK(launch_collide_stream(kStoreF32, pull, kVarReg4, gin, gout, p, kFullGrid, true, st));
+    CK(launch_ib_force(kStoreF32, pull, ctx->width, gin, p, q, true, st));
+    CK(launch_collide_stream(kStoreF32, pull, kVarReg2, gin, gout, p, kFullGrid, true, st));
     return BTDF_OK;
 }
 
@@ -891,14 +885,10 @@ int tape_backward_enqueue(btdf_ctx* ctx, cudaStream_t st) {
     CK(cudaMemsetAsync(T.lam[0], 0, sb, st));   // dJ/dg^N = 0
     AdjParams q{};
     q.nmark = nm;
-    q.nband = (int)ctx->band_keys.size();
     q.mk = ctx->d_mk;
     q.aux = ctx->d_aux;
     q.am = T.am;
     q.cscale = T.cscale;
-    q.band_keys = T.band_keys;
-    q.fbar_band = T.fbar_band;
-    q.Fbar_band = T.Fbar_band;
     q.mbar = T.mbar;
     q.objw = T.objw;
     q.dJdX = T.acc;
@@ -913,7 +903,6 @@ int tape_backward_enqueue(btdf_ctx* ctx, cudaStream_t st) {
         for (int64_t n = e - 1; n >= s; n--) {
             LatticeParams p = lattice_params(ctx, ctx->cur);
             p.F = T.Fall + (size_t)n * nm;
-            CK(cudaMemsetAsync(T.lam[1 - c], 0, sb, st));
             CK(launch_adjoint_step(tape_state(T, j, n), T.lam[c], T.lam[1 - c], p, q, ctx->width,
                                    tape_pull(T, n), st));
             c = 1 - c;
@@ -969,10 +958,10 @@ int tape_graph_launch(btdf_ctx* ctx, bool backward) {
 
 int tape_alloc(btdf_ctx* ctx, int nck, int every, int64_t nsteps) {
     AdjointTape& T = ctx->tape;
-    const int nm = ctx->nmark, nb = (int)ctx->band_keys.size();
+    const int nm = ctx->nmark;
     const size_t E = (size_t)9 * ctx->plane;
     if (T.ck && T.state_elems == E && T.cap_ck >= nck && T.cap_every >= every && T.cap_F >= nsteps &&
-        T.cap_mark == nm && T.cap_band == nb)
+        T.cap_mark == nm)
         return BTDF_OK;
     free_tape(ctx);
     T.state_elems = E;
@@ -999,9 +988,6 @@ int tape_alloc(btdf_ctx* ctx, int nck, int every, int64_t nsteps) {
     TA(T.am, (size_t)nm);
     TA(T.cscale, (size_t)nm);
     TA(T.objw, (size_t)nm);
-    TA(T.band_keys, (size_t)std::max(nb, 1));
-    TA(T.fbar_band, (size_t)std::max(nb, 1) * kSeg * 9);
-    TA(T.Fbar_band, (size_t)std::max(nb, 1) * kSeg);
     TA(T.mbar, (size_t)nm);
     TA(T.acc, (size_t)2 * nm + 1);
 #undef TA
@@ -1010,7 +996,6 @@ int tape_alloc(btdf_ctx* ctx, int nck, int every, int64_t nsteps) {
     T.cap_every = every;
     T.cap_F = nsteps;
     T.cap_mark = nm;
-    T.cap_band = nb;
     return BTDF_OK;
 }
 
@@ -1628,9 +1613,6 @@ int btdf_adjoint_forward(btdf_ctx* ctx, int64_t nsteps, int32_t every, int32_t b
     CK(cudaMemcpyAsync(T.am, am.data(), sizeof(AdjMarker) * nm, cudaMemcpyHostToDevice, st));
     CK(cudaMemcpyAsync(T.cscale, cscale.data(), sizeof(float) * nm, cudaMemcpyHostToDevice, st));
     CK(cudaMemcpyAsync(T.objw, objw.data(), sizeof(float2) * nm, cudaMemcpyHostToDevice, st));
-    if (!ctx->band_keys.empty())
-        CK(cudaMemcpyAsync(T.band_keys, ctx->band_keys.data(), sizeof(int) * ctx->band_keys.size(),
-                           cudaMemcpyHostToDevice, st));
 
     // forward window from the context's state, checkpoints every `every` steps
     CK(cudaMemcpyAsync(T.ck, ctx->g[ctx->cur], sizeof(float) * T.state_elems, cudaMemcpyDeviceToDevice, st));

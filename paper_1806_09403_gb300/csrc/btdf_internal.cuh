@@ -307,14 +307,11 @@ struct AdjMarker {
 };
 
 struct AdjParams {
-    int nmark, nband;
+    int nmark;
     const Marker* mk;
     const MarkerAux* aux;
     const AdjMarker* am;
     const float* cscale;       // drs * ds of each marker's body
-    const int* band_keys;      // [nband] y * nseg + segment
-    float* fbar_band;          // [nband * kSeg * 9] dJ/df parked at band nodes
-    float2* Fbar_band;         // [nband * kSeg] dJ/dF (node force) at band nodes
     float4* mbar;              // [nmark] (dJ/drho_l, dJ/dU*_l)
     const float2* objw;        // [nmark] explicit dJ/dF_l of the objective
     double* dJdX;              // [nmark] accumulated over the window
@@ -323,8 +320,8 @@ struct AdjParams {
 };
 
 // Launcher implemented in btdf_adjoint.cu: g = g^n (pull: post-collision,
-// else post-streaming), lam = dJ/dg^{n+1}, gbar = dJ/dg^n (zeroed by the
-// caller); p.F must hold the Lagrangian forces F^n of the step.
+// else post-streaming), lam = dJ/dg^{n+1}, gbar = dJ/dg^n (every entry is
+// written); p.F must hold the Lagrangian forces F^n of the step.
 cudaError_t launch_adjoint_step(const float* g, const float* lam, float* gbar, const LatticeParams& p,
                                 const AdjParams& q, int width, bool pull, cudaStream_t st);
 
