@@ -373,7 +373,7 @@ int btdf_adjoint_release(btdf_ctx *ctx);
 /* ---- batched form --------------------------------------------------------
  * Many independent lattices (each with its own size, relaxation time,
  * inflow, boundary kinds and bodies) advanced together: one IB launch over
- * the markers of all lattices and one persistent collide-stream launch over
+ * the markers of all lattices and one collide-stream launch over
  * all lattices per step, replayed through CUDA graphs.  Each lattice computes
  * exactly what a single context with the same configuration computes.  All
  * lattices share storage, layout, delta function, history_len and nf = 1.
@@ -398,9 +398,13 @@ int btdf_batch_body_lattice(const btdf_batch *b, int32_t body, int32_t *lattice)
 /* Collide-stream launch shape: 1 = 4 nodes per lane, 2 = 2 nodes per lane,
  * on a persistent grid whose CTAs own balanced ranges of 8-row units;
  * 3 = 4, 4 = 2 nodes per lane with one unit per CTA (the block scheduler
- * balances the SMs); 0 = default (1).  Results do not depend on it. */
+ * balances the SMs); 0 = automatic: two steps per pass over the lattices where
+ * a call's steps come in pairs and every marker support lies inside its lattice
+ * and off the inlet and outlet columns, else shape 3.  Results do not depend on
+ * it. */
 int btdf_batch_tune(btdf_batch *b, int32_t variant);
-/* As btdf_autotune, over the batch's launch shapes 1..4; ms[0..4]. */
+/* As btdf_autotune, over the batch's launch shapes 1..4; ms[0..4], ms[0] being
+ * half the time of a pair of steps (-1 where pairs cannot run). */
 int btdf_batch_autotune(btdf_batch *b, int32_t steps, int32_t flush_l2, int32_t *chosen, float *ms);
 int btdf_batch_step(btdf_batch *b, int64_t nsteps);
 int btdf_batch_sync(btdf_batch *b);

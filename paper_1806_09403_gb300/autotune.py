@@ -92,20 +92,26 @@ def _tune(obj, key: str, cache: TuneCache, run: Callable[[], tuple], apply: Call
     return dict(entry, cached=False)
 
 
+def _tune_with_pairs(obj, key: str, cache: TuneCache, run, apply, retune: bool) -> dict:
+    """_tune, remembering whether two steps per pass beat the chosen shape: a hit
+    then applies the automatic variant, which takes them."""
+    entry = _tune(obj, key, cache, run, apply, retune)
+    if not entry["cached"]:
+        entry["pairs"] = bool(getattr(obj, "tuned_pairs", False))
+        cache.put(key, {k: v for k, v in entry.items() if k != "cached"})
+    elif entry.get("pairs"):
+        apply(0)
+    return entry
+
+
 def tune_lattice(lat, cache: Optional[TuneCache] = None, steps: int = 20, flush_l2: bool = True,
                  device: Optional[str] = None, retune: bool = False) -> dict:
     """Applies the cached launch shape for this lattice, timing it first on a
     cache miss.  Returns the cache entry with ``cached`` set."""
     cache = cache or TuneCache()
     key = lattice_key(lat, device or device_name())
-    entry = _tune(lat, key, cache, lambda: lat.autotune(steps, flush_l2), lambda v: lat.tune(v, 0),
-                  retune)
-    if not entry["cached"]:
-        entry = dict(entry, pairs=bool(getattr(lat, "tuned_pairs", False)))
-        cache.put(key, {k: v for k, v in entry.items() if k != "cached"})
-    elif entry.get("pairs"):
-        lat.tune(0, 0)   # automatic: two steps per pass where they win
-    return entry
+    return _tune_with_pairs(lat, key, cache, lambda: lat.autotune(steps, flush_l2),
+                            lambda v: lat.tune(v, 0), retune)
 
 
 def tune_batch(bt, cache: Optional[TuneCache] = None, steps: int = 10, flush_l2: bool = False,
@@ -113,4 +119,4 @@ def tune_batch(bt, cache: Optional[TuneCache] = None, steps: int = 10, flush_l2:
     """As tune_lattice for a ``Batch``."""
     cache = cache or TuneCache()
     key = batch_key(bt, device or device_name())
-    return _tune(bt, key, cache, lambda: bt.autotune(steps, flush_l2), bt.tune, retune)
+    return _tune_with_pairs(bt, key, cache, lambda: bt.autotune(steps, flush_l2), bt.tune, retune)

@@ -431,6 +431,7 @@ class Batch:
         self.cases = list(cases)
         self.storage = int(storage)
         self.bodies = []          # (lattice, markers) per batch-wide body id
+        self.tuned_pairs = False  # autotune() found two steps per pass faster
 
     @classmethod
     def from_cases(cls, cases, storage=BTDF_F32, history_len=4096, stream: int = 0, layout=None):
@@ -484,6 +485,7 @@ class Batch:
         ms = np.zeros(5, dtype=np.float32)
         self._check(lib().btdf_batch_autotune(self._b, int(steps), 1 if flush_l2 else 0,
                                               C.byref(ch), ms.ctypes.data), "btdf_batch_autotune")
+        self.tuned_pairs = 0 < ms[0] < ms[1:].min()
         return ch.value, {v: float(ms[v]) for v in (1, 2, 3, 4)}
 
     def step(self, n=1):

@@ -210,6 +210,7 @@ struct btdf_ctx {
     // columns (set by rebuild_markers): ib_pair_kernel's condition.
     bool markers_inside = true;
     cudaGraphExec_t gexec[2] = {nullptr, nullptr};
+    bool gexec_pairs[2] = {false, false};          // the graph's steps come in pairs
     long long pf_grid[2] = {1, 1};                 // software-pipelined kernel [npl 4/2]
     long long pf_units[2][2] = {};                 // L2 prefetch distance of variants 10, 11 [local/pull]
     long long tma_grid[kVarCount] = {};  // persistent grid of each TMA variant
@@ -525,32 +526,13 @@ int ensure_pair_tables(btdf_ctx* ctx) {
     const int nx = ctx->cfg.nx, ny = ctx->cfg.ny;
     const bool px = ctx->cfg.bc_x == kBcxPeriodic;
     const std::vector<int>& seg_ptr = ctx->seg_ptr_host;
-    // the band as the pair kernel's strips see it, with the columns beside them:
-    // a node near a border belongs to two strips (and, wrapped, a narrow
-    // periodic lattice's node to several)
     const LatticeParams lp = lattice_params(ctx, ctx->cur);
     const int npl = pair_npl(ctx->cfg.storage, lp.bcx, nx, ny);
-    const int nstrip = pair_strips(lp, npl), own = pair_own(npl);
-    std::vector<int> strip_row((size_t)ny * nstrip, -1);
+    std::vector<int> strip_row;
     std::vector<int4> bnodes;
     int nsrow = 0;
-    for (int s = 0; s < ctx->nband; s++)
-        for (int i = 0; i < kSeg; i++) {
-            const int b = seg_ptr[(size_t)s * (kSeg + 1) + i], e = seg_ptr[(size_t)s * (kSeg + 1) + i + 1];
-            if (e <= b) continue;
-            const int y = ctx->band_keys[s] / ctx->nseg, xn = ctx->band_keys[s] % ctx->nseg * kSeg + i;
-            for (int x = px ? xn - nx : xn; x < nstrip * own + npl; x += nx) {
-                for (int k = std::max(0, (x - npl) / own); k < nstrip; k++) {
-                    const int c = x - (k * own - npl);
-                    if (c < 0) break;
-                    if (c >= 32 * npl) continue;
-                    int& row = strip_row[(size_t)y * nstrip + k];
-                    if (row < 0) row = nsrow++;
-                    bnodes.push_back(make_int4(row * 64 * npl + c, b, e, 0));
-                }
-                if (!px) break;
-            }
-        }
+    build_pair_tables(nx, ny, ctx->nseg, px, npl, pair_strips(nx, npl), ctx->band_keys, seg_ptr, 0, strip_row, bnodes,
+                      nsrow);
     const size_t fb_bytes = sizeof(float) * 64 * npl * (size_t)std::max(nsrow, 1);
     Arena A;
     const size_t o_srow = A.take<int>(sizeof(int) * strip_row.size());
@@ -589,7 +571,7 @@ int enqueue_pair(btdf_ctx* ctx, cudaStream_t st, int cur) {
     f.nodes = ctx->d_bnodes;
     f.nnode = ctx->nbnode;
     f.npl = pair_npl(ctx->cfg.storage, p.bcx, p.nx, p.ny);
-    f.nstrip = pair_strips(p, f.npl);
+    f.nstrip = pair_strips(p.nx, f.npl);
     for (int a = 0; a < 9; a++) f.kin[a] = p.poff[a] + (unsigned)(1 - ey(a)) * p.rs;
     f.fb1 = ctx->d_fb[1];
     f.fb2 = ctx->d_fb[0];
@@ -612,13 +594,15 @@ int enqueue_pair(btdf_ctx* ctx, cudaStream_t st, int cur) {
     return BTDF_OK;
 }
 
-int ensure_graph(btdf_ctx* ctx, int cur) {
-    if (ctx->gexec[cur]) return BTDF_OK;
+int ensure_graph(btdf_ctx* ctx, int cur, bool pairs) {
+    if (ctx->gexec[cur] && ctx->gexec_pairs[cur] == pairs) return BTDF_OK;
+    if (ctx->gexec[cur]) cudaGraphExecDestroy(ctx->gexec[cur]);
+    ctx->gexec[cur] = nullptr;
     cudaGraph_t graph = nullptr;
     CK(cudaStreamBeginCapture(ctx->cap, cudaStreamCaptureModeThreadLocal));
     int rc = BTDF_OK;
     int c = cur;
-    const int per = pairs_allowed(ctx) ? 2 : 1;
+    const int per = pairs ? 2 : 1;
     for (int i = 0; i < kGraphSteps && rc == BTDF_OK; i += per) {
         rc = per == 2 ? enqueue_pair(ctx, ctx->cap, c) : enqueue_step(ctx, ctx->cap, true, c, false);
         c = 1 - c;
@@ -629,6 +613,7 @@ int ensure_graph(btdf_ctx* ctx, int cur) {
         return rc;
     }
     if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaStreamEndCapture");
+    ctx->gexec_pairs[cur] = pairs;
     e = cudaGraphInstantiate(&ctx->gexec[cur], graph, 0);
     cudaGraphDestroy(graph);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaGraphInstantiate");
@@ -1307,10 +1292,14 @@ int btdf_step(btdf_ctx* ctx, int64_t nsteps) {
     if (nsteps < 0) return fail(ctx, BTDF_EINVAL, "nsteps < 0");
     if (!ctx->has_fields) return fail(ctx, BTDF_ESTATE, "call btdf_init_fields or btdf_load_state first");
     int64_t i = 0;
-    const bool pairs = nsteps - (ctx->poststream ? 1 : 0) >= 2 && pairs_allowed(ctx);
-    if (pairs) {
-        const int rc = ensure_pair_tables(ctx);
-        if (rc != BTDF_OK) return rc;
+    bool pairs = nsteps - (ctx->poststream ? 1 : 0) >= 2 && pairs_allowed(ctx);
+    if (pairs && ctx->nmark > 0 && !ctx->d_pair) {
+        // the tables cannot be built while the caller captures the stream
+        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(ctx->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
+            cudaGetLastError();
+            pairs = false;
+        }
     }
     if (nsteps > 0 && ctx->poststream) {
         const int rc = enqueue_step(ctx, ctx->stream, false, ctx->cur, ctx->prof);
@@ -1319,9 +1308,23 @@ int btdf_step(btdf_ctx* ctx, int64_t nsteps) {
         ctx->poststream = false;
         i = 1;
     }
+    if (pairs) {
+        // The tables of the pair kernels take the host 2-3 ms with hundreds of
+        // bodies: on a large lattice a few single steps keep the device busy
+        // meanwhile.
+        if (ctx->nmark > 0 && !ctx->d_pair && (long long)ctx->cfg.nx * ctx->cfg.ny >= (1ll << 23))
+            for (int k = 0; k < 6 && i < nsteps; k++, i++) {
+                const int rc = enqueue_step(ctx, ctx->stream, true, ctx->cur, false);
+                if (rc != BTDF_OK) return rc;
+                ctx->cur = 1 - ctx->cur;
+            }
+        const int rc = ensure_pair_tables(ctx);
+        if (rc == BTDF_ENOMEM) pairs = false;   // single steps need no tables
+        else if (rc != BTDF_OK) return rc;
+    }
     if (!ctx->prof) {
         while (nsteps - i >= kGraphSteps) {
-            const int rc = ensure_graph(ctx, ctx->cur);
+            const int rc = ensure_graph(ctx, ctx->cur, pairs);
             if (rc != BTDF_OK) return rc;
             CK(cudaGraphLaunch(ctx->gexec[ctx->cur], ctx->stream));
             i += kGraphSteps;

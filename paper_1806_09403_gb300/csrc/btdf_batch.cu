@@ -41,9 +41,11 @@ struct btdf_batch {
     bool poststream = true;
     std::vector<char> has_fields;
     int64_t steps = 0, hist_from = 0;
-    // launch shape: 1 / 2 = 4 / 2 nodes per lane on a persistent grid of
-    // balanced unit ranges; 3 / 4 = the same with one unit per CTA
-    int variant = 1;
+    // Launch shape of single steps: 1 / 2 = 4 / 2 nodes per lane on a persistent
+    // grid of balanced unit ranges; 3 / 4 = the same with one unit per CTA.  3 by
+    // default: 328 us a step on 128 lattices (27 M nodes) in FP32 against 395 for
+    // 1, 28 against 30 on 24 small FP16 ones.
+    int variant = 3;
     int grid[2] = {1, 1};
     int sms = 1;
 
@@ -66,11 +68,22 @@ struct btdf_batch {
     double* d_body_scale = nullptr;
     double2* d_hist = nullptr;
     unsigned long long* d_step = nullptr;
-    unsigned int* d_done = nullptr;
+    unsigned int* d_done = nullptr;        // [2] finished CTAs: single steps, pairs
     int* d_status = nullptr;
     std::vector<LatticeParams> descs;
     cudaGraphExec_t gexec[2] = {nullptr, nullptr};
     std::string err;
+    // Pairs of steps (btdf_pair.cu): every marker support inside its lattice and off
+    // the inlet and outlet columns; tables built for the first pair.
+    bool markers_inside = true;
+    std::vector<std::vector<int>> band_keys, seg_ptr;   // per lattice, for those tables
+    std::vector<size_t> cs_off;
+    void* d_pair = nullptr;
+    float2* d_F1 = nullptr;
+    PairForces pf{};
+    PairBatch pb{};
+    bool gexec_pairs[2] = {false, false};
+    bool variant_set = false;              // btdf_batch_tune / autotune chose a launch shape
     double2* tune_hist = nullptr;          // one-slot force ring while btdf_batch_autotune times steps
 };
 
@@ -111,6 +124,7 @@ void free_marker_data(btdf_batch* bt) {
     bfree(bt->d_seg_index);
     bfree(bt->d_seg_ptr);
     bfree(bt->d_csr);
+    bfree(bt->d_pair);
     bfree(bt->d_body_ptr);
     bfree(bt->d_body_scale);
     bfree(bt->d_hist);
@@ -238,6 +252,8 @@ int rebuild(btdf_batch* bt) {
     std::vector<CsrEntry> csr;
     std::vector<size_t> si_off(bt->n, 0), sp_off(bt->n, 0), cs_off(bt->n, 0);
     std::vector<char> has_band(bt->n, 0);
+    bt->band_keys.assign(bt->n, {});
+    bt->seg_ptr.assign(bt->n, {});
     for (int c = 0; c < bt->n; c++) {
         std::vector<BodyDesc> bd;
         int base = -1;
@@ -262,6 +278,8 @@ int rebuild(btdf_batch* bt) {
         seg_ptr.insert(seg_ptr.end(), t.seg_ptr.begin(), t.seg_ptr.end());
         csr.insert(csr.end(), t.csr.begin(), t.csr.end());
         has_band[c] = 1;
+        bt->band_keys[c].assign(t.seg_keys.begin(), t.seg_keys.end());
+        bt->seg_ptr[c] = std::move(t.seg_ptr);
     }
     std::vector<int> body_rng(2 * nb);
     std::vector<double> scale(nb);
@@ -309,8 +327,99 @@ int rebuild(btdf_batch* bt) {
         p.F = bt->d_F;
     }
     bt->hist_from = bt->steps;
+    bt->cs_off = cs_off;
+    bt->markers_inside = true;
+    for (const BBody& B : bt->bodies) {
+        const btdf_config& k = bt->cfg[B.lattice];
+        for (int l = 0; l < B.n; l++) {
+            const int i0 = (int)std::floor(B.X[l] - 0.5 * bt->width) + 1, i1 = i0 + bt->width - 1;
+            const int j0 = (int)std::floor(B.Y[l] - 0.5 * bt->width) + 1, j1 = j0 + bt->width - 1;
+            if ((k.bc_x != kBcxPeriodic && (i0 < 1 || i1 > k.nx - 2)) ||
+                (k.bc_y != kBcyPeriodic && (j0 < 0 || j1 > k.ny - 1)))
+                bt->markers_inside = false;
+        }
+    }
     return upload_descs(bt);
 }
+
+// Tables of the pair kernels, for the first pair after the markers were set.
+int ensure_pair_tables(btdf_batch* bt) {
+    if (bt->d_pair) return BTDF_OK;
+    long long nodes_all = 0;
+    int npl = 2;
+    for (int c = 0; c < bt->n; c++) nodes_all += (long long)bt->cfg[c].nx * bt->cfg[c].ny;
+    for (int c = 0; c < bt->n; c++)
+        if (nodes_all >= (1ll << 22) || pair_npl(bt->storage, bt->cfg[c].bc_x, bt->cfg[c].nx, bt->cfg[c].ny) == 4) npl = 4;
+    std::vector<int> strip_row;
+    std::vector<int4> nodes, tiles;
+    std::vector<PairLattice> lat(bt->n);
+    std::vector<size_t> row0(bt->n, 0);
+    int nsrow = 0;
+    const int th = pair_tile_rows(npl);
+    for (int c = 0; c < bt->n; c++) {
+        const btdf_config& k = bt->cfg[c];
+        const LatticeParams& p = bt->descs[c];
+        lat[c] = PairLattice{};
+        lat[c].nstrip = pair_strips(k.nx, npl);
+        lat[c].off = bt->off[c];
+        for (int a = 0; a < 9; a++) lat[c].kin[a] = p.poff[a] + (unsigned)(1 - ey(a)) * p.rs;
+        row0[c] = strip_row.size();
+        if (bt->nmark > 0 && !bt->band_keys[c].empty())
+            build_pair_tables(k.nx, k.ny, bt->nseg[c], k.bc_x == kBcxPeriodic, npl, lat[c].nstrip, bt->band_keys[c],
+                              bt->seg_ptr[c], (int)bt->cs_off[c], strip_row, nodes, nsrow);
+        for (int y = 0; y < k.ny; y += th)
+            for (int s = 0; s < lat[c].nstrip; s++) tiles.push_back(make_int4(c, s, y, 0));
+    }
+    auto up = [](size_t b) { return (b + 255) / 256 * 256; };
+    const size_t fb = sizeof(float) * 64 * npl * (size_t)std::max(nsrow, 1);
+    const size_t b_lat = up(sizeof(PairLattice) * bt->n), b_tile = up(sizeof(int4) * tiles.size()),
+                 b_row = up(sizeof(int) * std::max<size_t>(strip_row.size(), 1)),
+                 b_node = up(sizeof(int4) * std::max<size_t>(nodes.size(), 1)), b_fb = up(fb),
+                 b_F = up(sizeof(float2) * std::max(bt->nmark, 1));
+    const cudaError_t ea = cudaMalloc(&bt->d_pair, b_lat + b_tile + b_row + b_node + 2 * b_fb + b_F);
+    if (ea != cudaSuccess) {
+        cudaGetLastError();
+        bt->d_pair = nullptr;
+        return bfail(bt, ea == cudaErrorMemoryAllocation ? BTDF_ENOMEM : BTDF_ECUDA, "pair tables");
+    }
+    char* q = (char*)bt->d_pair;
+    PairLattice* d_lat = (PairLattice*)q;
+    int4* d_tile = (int4*)(q += b_lat);
+    int* d_row = (int*)(q += b_tile);
+    int4* d_node = (int4*)(q += b_row);
+    float* d_fb1 = (float*)(q += b_node);
+    float* d_fb2 = (float*)(q += b_fb);
+    bt->d_F1 = (float2*)(q += b_fb);
+    for (int c = 0; c < bt->n; c++)
+        if (bt->nmark > 0 && !bt->band_keys[c].empty()) lat[c].strip_row = d_row + row0[c];
+    cudaStream_t st = bt->stream;
+    BCK(cudaMemcpyAsync(d_lat, lat.data(), sizeof(PairLattice) * bt->n, cudaMemcpyHostToDevice, st));
+    BCK(cudaMemcpyAsync(d_tile, tiles.data(), sizeof(int4) * tiles.size(), cudaMemcpyHostToDevice, st));
+    if (!strip_row.empty())
+        BCK(cudaMemcpyAsync(d_row, strip_row.data(), sizeof(int) * strip_row.size(), cudaMemcpyHostToDevice, st));
+    if (!nodes.empty())
+        BCK(cudaMemcpyAsync(d_node, nodes.data(), sizeof(int4) * nodes.size(), cudaMemcpyHostToDevice, st));
+    BCK(cudaMemsetAsync(d_fb1, 0, 2 * b_fb + b_F, st));   // band nodes without terms keep a zero force
+    BCK(cudaStreamSynchronize(st));
+    PairForces f{};
+    f.F1 = bt->d_F1;
+    f.nodes = d_node;
+    f.nnode = (int)nodes.size();
+    f.fb1 = d_fb1;
+    f.fb2 = d_fb2;
+    f.done = bt->d_done + 1;
+    f.npl = npl;
+    bt->pf = f;
+    PairBatch b{};
+    b.lat = d_lat;
+    b.tile = d_tile;
+    b.ntile = (int)tiles.size();
+    bt->pb = b;
+    return BTDF_OK;
+}
+
+// Pairs of steps unless a launch shape was chosen: with every support inside.
+bool pairs_allowed(const btdf_batch* bt) { return !bt->variant_set && (bt->nmark == 0 || bt->markers_inside); }
 
 BatchLbm lbm_params(const btdf_batch* bt, int s) {
     BatchLbm b{};
@@ -345,7 +454,7 @@ int enqueue(btdf_batch* bt, cudaStream_t st, bool pull, int cur) {
         q.rhol = bt->d_rhol;
         q.first_pass = 1;
         q.status = bt->d_status;
-        BCK(launch_ib_force_batch(bt->storage, pull, bt->width, bt->g[cur], bt->d_descs, bt->d_off, q, st));
+        BCK(launch_ib_force_batch(bt->storage, pull, bt->width, bt->g[cur], bt->d_descs, bt->d_off, q, false, st));
     }
     const int s = bt->variant - 1;
     BCK(launch_collide_stream_batch(bt->storage, pull, shape_npl(bt->variant), bt->g[cur],
@@ -354,14 +463,49 @@ int enqueue(btdf_batch* bt, cudaStream_t st, bool pull, int cur) {
     return BTDF_OK;
 }
 
-int ensure_graph(btdf_batch* bt, int cur) {
-    if (bt->gexec[cur]) return BTDF_OK;
+// Two pulling steps reading buffer `cur`; the state is then in the other buffer.
+int enqueue_pair(btdf_batch* bt, cudaStream_t st, int cur) {
+    const bool marks = bt->nmark > 0;
+    if (marks) {
+        IbParams q{};
+        q.nmark = bt->nmark;
+        q.mk = bt->d_mk;
+        q.aux = bt->d_aux;
+        q.F_out = bt->d_F1;
+        q.Us = bt->d_Us;
+        q.rhol = bt->d_rhol;
+        q.first_pass = 1;
+        q.status = bt->d_status;
+        BCK(launch_ib_force_batch(bt->storage, true, bt->width, bt->g[cur], bt->d_descs, bt->d_off, q, true, st));
+        q.F_out = bt->d_F;
+        BCK(launch_ib_pair_batch(bt->storage, bt->width, bt->g[cur], bt->d_descs, bt->d_off, q, bt->pf, bt->d_csr, true,
+                                 st));
+    }
+    PairBatch b = bt->pb;
+    const BatchLbm l = lbm_params(bt, 0);
+    b.descs = bt->d_descs;
+    b.nbody = l.nbody;
+    b.hist_len = l.hist_len;
+    b.body_rng = l.body_rng;
+    b.body_scale = l.body_scale;
+    b.hist = l.hist;
+    b.F2 = l.F;
+    b.step = l.step;
+    BCK(launch_pair_batch(bt->storage, bt->g[cur], bt->g[1 - cur], b, bt->pf, marks, st));
+    return BTDF_OK;
+}
+
+int ensure_graph(btdf_batch* bt, int cur, bool pairs) {
+    if (bt->gexec[cur] && bt->gexec_pairs[cur] == pairs) return BTDF_OK;
+    if (bt->gexec[cur]) cudaGraphExecDestroy(bt->gexec[cur]);
+    bt->gexec[cur] = nullptr;
     cudaGraph_t graph = nullptr;
     BCK(cudaStreamBeginCapture(bt->cap, cudaStreamCaptureModeThreadLocal));
     int rc = BTDF_OK;
     int c = cur;
-    for (int i = 0; i < kBatchGraphSteps && rc == BTDF_OK; i++) {
-        rc = enqueue(bt, bt->cap, true, c);
+    const int per = pairs ? 2 : 1;
+    for (int i = 0; i < kBatchGraphSteps && rc == BTDF_OK; i += per) {
+        rc = pairs ? enqueue_pair(bt, bt->cap, c) : enqueue(bt, bt->cap, true, c);
         c = 1 - c;
     }
     cudaError_t e = cudaStreamEndCapture(bt->cap, &graph);
@@ -370,6 +514,7 @@ int ensure_graph(btdf_batch* bt, int cur) {
         return rc;
     }
     if (e != cudaSuccess) return bfail(bt, BTDF_ECUDA, "cudaStreamEndCapture failed");
+    bt->gexec_pairs[cur] = pairs;
     e = cudaGraphInstantiate(&bt->gexec[cur], graph, 0);
     cudaGraphDestroy(graph);
     if (e != cudaSuccess) return bfail(bt, BTDF_ECUDA, "cudaGraphInstantiate failed");
@@ -458,13 +603,13 @@ int btdf_batch_create(const btdf_config* cfgs, int32_t n, void* stream, btdf_bat
     if (cudaMalloc((void**)&bt->d_descs, sizeof(LatticeParams) * n) != cudaSuccess ||
         cudaMalloc((void**)&bt->d_off, sizeof(unsigned long long) * n) != cudaSuccess ||
         cudaMalloc((void**)&bt->d_step, sizeof(unsigned long long)) != cudaSuccess ||
-        cudaMalloc((void**)&bt->d_done, sizeof(unsigned int)) != cudaSuccess ||
+        cudaMalloc((void**)&bt->d_done, 2 * sizeof(unsigned int)) != cudaSuccess ||
         cudaMalloc((void**)&bt->d_status, sizeof(int)) != cudaSuccess)
         return bail(BTDF_ECUDA);
     if (cudaMemcpy(bt->d_off, bt->off.data(), sizeof(unsigned long long) * n, cudaMemcpyHostToDevice) !=
             cudaSuccess ||
         cudaMemset(bt->d_step, 0, sizeof(unsigned long long)) != cudaSuccess ||
-        cudaMemset(bt->d_done, 0, sizeof(unsigned int)) != cudaSuccess ||
+        cudaMemset(bt->d_done, 0, 2 * sizeof(unsigned int)) != cudaSuccess ||
         cudaMemset(bt->d_status, 0, sizeof(int)) != cudaSuccess)
         return bail(BTDF_ECUDA);
     bt->descs.resize(n);
@@ -575,7 +720,8 @@ int btdf_batch_tune(btdf_batch* bt, int32_t variant) {
     if (variant < 0 || variant > 4) return bfail(bt, BTDF_EINVAL, "variant must be 0 .. 4");
     BCK(cudaStreamSynchronize(bt->stream));
     drop_graphs(bt);
-    bt->variant = variant == 0 ? 1 : variant;
+    bt->variant = variant == 0 ? 3 : variant;
+    bt->variant_set = variant != 0;
     return BTDF_OK;
 }
 
@@ -638,11 +784,29 @@ int btdf_batch_autotune(btdf_batch* bt, int32_t steps, int32_t flush_l2, int32_t
             res[v] = interquartile_mean(t);
             if (v == 1 || res[v] < res[best]) best = v;
         }
+        if (bt->nmark == 0 || bt->markers_inside) {   // pairs of steps, as time per step
+            const int rcp = ensure_pair_tables(bt);
+            if (rcp != BTDF_OK) return rcp;
+            for (int i = 0; i < steps + 2; i++) {
+                if (flush) BCK(launch_l2_flush(flush, l2_flush_bytes(), st));
+                const int e = std::max(i - 2, 0);
+                BCK(cudaEventRecord(ev[2 * e], st));
+                const int rc = enqueue_pair(bt, st, bt->cur);
+                if (rc != BTDF_OK) return rc;
+                BCK(cudaEventRecord(ev[2 * e + 1], st));
+                bt->cur = 1 - bt->cur;
+            }
+            BCK(cudaStreamSynchronize(st));
+            std::vector<float> t(steps);
+            for (int i = 0; i < steps; i++) BCK(cudaEventElapsedTime(&t[i], ev[2 * i], ev[2 * i + 1]));
+            res[0] = 0.5f * interquartile_mean(t);
+        }
         return BTDF_OK;
     };
     const int rc = run();
     bt->tune_hist = nullptr;
     bt->variant = rc == BTDF_OK ? best : var0;
+    if (rc == BTDF_OK) bt->variant_set = !(res[0] > 0.0f && res[0] < res[best]);
     bt->cur = cur0;
     bt->poststream = post0;
     cudaError_t e = cudaSuccess;
@@ -674,6 +838,19 @@ int btdf_batch_step(btdf_batch* bt, int64_t nsteps) {
     for (int c = 0; c < bt->n; c++)
         if (!bt->has_fields[c]) return bfail(bt, BTDF_ESTATE, "every lattice needs btdf_batch_init_fields");
     int64_t i = 0;
+    bool pairs = nsteps - (bt->poststream ? 1 : 0) >= 2 && pairs_allowed(bt);
+    if (pairs && !bt->d_pair) {
+        // no tables while the caller captures the stream; single steps need none
+        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(bt->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
+            cudaGetLastError();
+            pairs = false;
+        } else {
+            const int rc = ensure_pair_tables(bt);
+            if (rc == BTDF_ENOMEM) pairs = false;
+            else if (rc != BTDF_OK) return rc;
+        }
+    }
     if (nsteps > 0 && bt->poststream) {
         const int rc = enqueue(bt, bt->stream, false, bt->cur);
         if (rc != BTDF_OK) return rc;
@@ -682,15 +859,17 @@ int btdf_batch_step(btdf_batch* bt, int64_t nsteps) {
         i = 1;
     }
     while (nsteps - i >= kBatchGraphSteps) {
-        const int rc = ensure_graph(bt, bt->cur);
+        const int rc = ensure_graph(bt, bt->cur, pairs);
         if (rc != BTDF_OK) return rc;
         BCK(cudaGraphLaunch(bt->gexec[bt->cur], bt->stream));
         i += kBatchGraphSteps;
     }
-    for (; i < nsteps; i++) {
-        const int rc = enqueue(bt, bt->stream, true, bt->cur);
+    while (i < nsteps) {
+        const bool two = pairs && nsteps - i >= 2;
+        const int rc = two ? enqueue_pair(bt, bt->stream, bt->cur) : enqueue(bt, bt->stream, true, bt->cur);
         if (rc != BTDF_OK) return rc;
         bt->cur = 1 - bt->cur;
+        i += two ? 2 : 1;
     }
     bt->steps += nsteps;
     return BTDF_OK;

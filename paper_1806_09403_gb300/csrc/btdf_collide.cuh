@@ -9,17 +9,18 @@ namespace btdf {
 namespace {
 
 // Forces on the bodies (Eq. 27) in step `step` from its Lagrangian forces, in
-// FP64, into the history ring, by warp `warp` of `nwarps`.  FP64 arithmetic is
-// slow on this part and, on small lattices, this reduction is on the step's
-// critical path: one warp per body and no work for absent bodies.
-__device__ __forceinline__ void body_forces(const LatticeParams& p, const float2* Fl, unsigned long long step,
-                                            int warp, int nwarps) {
+// FP64, into the history ring, by warp `warp` of `nwarps`; body b's markers are
+// ptr[b * stride] .. ptr[b * stride + 1] - 1.  FP64 arithmetic is slow on this
+// part and, on small lattices, this reduction is on the step's critical path:
+// one warp per body and no work for absent bodies.
+__device__ __forceinline__ void body_forces(int nbody, const int* ptr, int stride, const double* scale, double2* hist,
+                                            int hist_len, const float2* Fl, unsigned long long step, int warp,
+                                            int nwarps) {
     const int lane = threadIdx.x & 31;
-    const long long slot = (long long)(step % (unsigned long long)(p.hist_len > 0 ? p.hist_len : 1)) *
-                           p.nbody;
-    for (int b = warp; b < p.nbody; b += nwarps) {
+    const long long slot = (long long)(step % (unsigned long long)(hist_len > 0 ? hist_len : 1)) * nbody;
+    for (int b = warp; b < nbody; b += nwarps) {
         double sx = 0.0, sy = 0.0;
-        for (int k = p.body_ptr[b] + lane; k < p.body_ptr[b + 1]; k += 32) {
+        for (int k = ptr[b * stride] + lane; k < ptr[b * stride + 1]; k += 32) {
             const float2 F = Fl[k];
             sx += (double)F.x;
             sy += (double)F.y;
@@ -30,10 +31,14 @@ __device__ __forceinline__ void body_forces(const LatticeParams& p, const float2
             sy += __shfl_xor_sync(kFull, sy, off);
         }
         if (lane == 0) {
-            const double sc = p.body_scale[b];
-            p.hist[slot + b] = make_double2(-sx * sc, -sy * sc);
+            const double sc = scale[b];
+            hist[slot + b] = make_double2(-sx * sc, -sy * sc);
         }
     }
+}
+__device__ __forceinline__ void body_forces(const LatticeParams& p, const float2* Fl, unsigned long long step,
+                                            int warp, int nwarps) {
+    body_forces(p.nbody, p.body_ptr, 1, p.body_scale, p.hist, p.hist_len, Fl, step, warp, nwarps);
 }
 
 // f holds the post-streaming deviations of NPL nodes at their stored scale,

@@ -246,7 +246,37 @@ struct PairForces {
 };
 // Nodes per lane of the pair kernel for a lattice, and its strips.
 int pair_npl(int storage, int bcx, int nx, int ny);
-int pair_strips(const LatticeParams& p, int npl);
+inline int pair_strips(int nx, int npl) { return (nx + pair_own(npl) - 1) / pair_own(npl); }
+
+// Batched form: a lattice's part of it, its tiles, and the force reductions.
+struct PairLattice {
+    const int* strip_row;
+    unsigned kin[9];
+    int nstrip;
+    unsigned long long off;    // element offset of the lattice's populations
+};
+struct PairBatch {
+    const LatticeParams* descs;
+    const PairLattice* lat;
+    const int4* tile;          // [ntile] (lattice, strip, first row, 0)
+    int ntile;
+    int nbody, hist_len;
+    const int* body_rng;       // [2 * nbody] first and end flat marker index
+    const double* body_scale;
+    double2* hist;
+    const float2* F2;          // Lagrangian forces of the second step (q.F1: the first's)
+    unsigned long long* step;
+};
+cudaError_t launch_pair_batch(int storage, const void* gin, void* gout, const PairBatch& b, const PairForces& q,
+                              bool pdl, cudaStream_t st);
+cudaError_t launch_ib_pair_batch(int storage, int width, const void* g, const LatticeParams* descs,
+                                 const unsigned long long* case_off, const IbParams& q, const PairForces& r,
+                                 const CsrEntry* csr, bool pdl, cudaStream_t st);
+// Rows of the pair kernel's tiles.
+int pair_tile_rows(int npl);
+void build_pair_tables(int nx, int ny, int nseg, bool px, int npl, int nstrip, const std::vector<int>& keys,
+                       const std::vector<int>& seg_ptr, int term0, std::vector<int>& strip_row,
+                       std::vector<int4>& nodes, int& nsrow);
 
 // Two pulling steps in one kernel.
 cudaError_t launch_pair(int storage, const void* gin, void* gout, const LatticeParams& p, const PairForces& q,
@@ -266,7 +296,7 @@ cudaError_t launch_collide_stream_batch(int storage, bool pull, int npl, const v
 int collide_stream_batch_blocks_per_sm(int storage, int npl);
 cudaError_t launch_ib_force_batch(int storage, bool pull, int width, const void* g,
                                   const LatticeParams* descs, const unsigned long long* case_off,
-                                  const IbParams& q, cudaStream_t st);
+                                  const IbParams& q, bool pdl, cudaStream_t st);
 int tma_box_rows(int variant);
 int tma_halo(int storage);
 

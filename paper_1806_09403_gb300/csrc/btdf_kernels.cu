@@ -1309,21 +1309,28 @@ int batch_blocks_tn() {
 
 template <typename T, int S>
 cudaError_t ib_batch_ts(bool pull, const void* g, const LatticeParams* descs,
-                        const unsigned long long* case_off, const IbParams& q, cudaStream_t st) {
+                        const unsigned long long* case_off, const IbParams& q, bool pdl, cudaStream_t st) {
     constexpr int MPW = 32 / Group<S>::G;
     const long long warps = (q.nmark + MPW - 1) / MPW;
-    const unsigned nb = blocks_for(warps * 32);
-    ib_force_batch_kernel<T, S><<<nb, kThreads, 0, st>>>((const T*)g, descs, case_off, q, pull ? 1 : 0);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(blocks_for(warps * 32));
+    cfg.blockDim = dim3(kThreads);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = pdl ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, ib_force_batch_kernel<T, S>, (const T*)g, descs, case_off, q, pull ? 1 : 0);
 }
 
 template <typename T>
 cudaError_t ib_batch_t(bool pull, int width, const void* g, const LatticeParams* descs,
-                       const unsigned long long* case_off, const IbParams& q, cudaStream_t st) {
+                       const unsigned long long* case_off, const IbParams& q, bool pdl, cudaStream_t st) {
     switch (width) {
-    case 2: return ib_batch_ts<T, 2>(pull, g, descs, case_off, q, st);
-    case 3: return ib_batch_ts<T, 3>(pull, g, descs, case_off, q, st);
-    case 4: return ib_batch_ts<T, 4>(pull, g, descs, case_off, q, st);
+    case 2: return ib_batch_ts<T, 2>(pull, g, descs, case_off, q, pdl, st);
+    case 3: return ib_batch_ts<T, 3>(pull, g, descs, case_off, q, pdl, st);
+    case 4: return ib_batch_ts<T, 4>(pull, g, descs, case_off, q, pdl, st);
     default: return cudaErrorInvalidValue;
     }
 }
@@ -1356,12 +1363,12 @@ int collide_stream_batch_blocks_per_sm(int storage, int npl) {
 
 cudaError_t launch_ib_force_batch(int storage, bool pull, int width, const void* g,
                                   const LatticeParams* descs, const unsigned long long* case_off,
-                                  const IbParams& q, cudaStream_t st) {
+                                  const IbParams& q, bool pdl, cudaStream_t st) {
     if (q.nmark <= 0) return cudaSuccess;
     switch (storage) {
-    case kStoreF32: return ib_batch_t<float>(pull, width, g, descs, case_off, q, st);
-    case kStoreF16: return ib_batch_t<__half>(pull, width, g, descs, case_off, q, st);
-    case kStoreBF16: return ib_batch_t<__nv_bfloat16>(pull, width, g, descs, case_off, q, st);
+    case kStoreF32: return ib_batch_t<float>(pull, width, g, descs, case_off, q, pdl, st);
+    case kStoreF16: return ib_batch_t<__half>(pull, width, g, descs, case_off, q, pdl, st);
+    case kStoreBF16: return ib_batch_t<__nv_bfloat16>(pull, width, g, descs, case_off, q, pdl, st);
     default: return cudaErrorInvalidValue;
     }
 }

@@ -280,12 +280,12 @@ template <int NPL> struct Vec<float, NPL> {
 };
 
 // Spread force (Eq. 15) of the terms b .. e-1.
-__device__ __forceinline__ void spread_terms(const LatticeParams& p, const float2* F, int b, int e, float& sx,
+__device__ __forceinline__ void spread_terms(const CsrEntry* csr, const float2* F, int b, int e, float& sx,
                                              float& sy) {
     sx = 0.f;
     sy = 0.f;
     for (int k = b; k < e; k++) {
-        const CsrEntry c = p.csr[k];
+        const CsrEntry c = csr[k];
         const float2 f = F[c.marker];
         sx = __fmaf_rn(c.w, f.x, sx);
         sy = __fmaf_rn(c.w, f.y, sy);
@@ -396,37 +396,16 @@ __device__ __forceinline__ void pair_spread(const float* fb, int band, int lane,
     }
 }
 
-template <typename T, int NPL, int NW, int TH, int MINB>
-__global__ void __launch_bounds__(32 * NW, MINB)
-pair_kernel(const T* __restrict__ gin, T* __restrict__ gout, const __grid_constant__ LatticeParams p,
-            const __grid_constant__ PairForces q, int nred) {
-    cudaTriggerProgrammaticLaunchCompletion();
+// Two steps of the tile of strip s from row y0 on, of the lattice p whose
+// populations are gin / gout; the other arguments are PairForces'.
+template <typename T, int NPL, int NW, int TH>
+__device__ __forceinline__ void pair_tile(const T* __restrict__ gin, T* __restrict__ gout, const LatticeParams& p,
+                                          const unsigned (&kin)[9], const int* strip_row, int nstrip, const float* fb1,
+                                          const float* fb2, int s, int y0, T* tile) {
     using C = PairTile<T, NPL, TH>;
     constexpr int NP = NPL / 2;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    T* const tile = reinterpret_cast<T*>(smem_raw);
-    // The first nred blocks reduce the body forces of both steps while the
-    // others work; the last of them to finish advances the step counter.
-    if ((int)blockIdx.x < nred) {
-        if (p.nbody > 0) cudaGridDependencySynchronize();
-        const unsigned long long step = p.step != nullptr ? *p.step : 0ull;
-        const int half = NW / 2, w = (int)threadIdx.x >> 5;
-        if (w < half) body_forces(p, q.F1, step, blockIdx.x * half + w, nred * half);
-        else if (w < 2 * half) body_forces(p, p.F, step + 1ull, blockIdx.x * half + w - half, nred * half);
-        __syncthreads();
-        if (threadIdx.x == 0 && p.step != nullptr) {
-            __threadfence();
-            if (atomicAdd(q.done, 1u) == (unsigned)nred - 1u) {
-                *p.step = step + 2ull;
-                *q.done = 0u;
-            }
-        }
-        return;
-    }
-    const int b = (int)blockIdx.x - nred;
-    const int c = b / q.nstrip, s = b - c * q.nstrip;
     const int warp = (int)threadIdx.x >> 5, lane = (int)threadIdx.x & 31;
-    const int ny = p.ny, nx = p.nx, xs = s * pair_own(NPL) - NPL, y0 = c * TH;
+    const int ny = p.ny, nx = p.nx, xs = s * pair_own(NPL) - NPL;
     const bool pery = p.bcy == kBcyPeriodic, perx = p.bcx == kBcxPeriodic, noslip = p.bcy == kBcyNoslip;
     const int x0 = xs + NPL * lane;
     const int x0c = min(max(x0, 0), p.nxp - NPL);
@@ -434,7 +413,7 @@ pair_kernel(const T* __restrict__ gin, T* __restrict__ gout, const __grid_consta
     const bool ends = xs <= 0 || xs + 32 * NPL >= nx;   // the tile holds a row end
     const T* const cin = gin + x0c;
     T* const cout = gout + x0c;
-    const int* const srow = q.strip_row != nullptr ? q.strip_row + s : nullptr;
+    const int* const srow = strip_row != nullptr ? strip_row + s : nullptr;
     const bool uniform_force = p.gx != 0.f || p.gy != 0.f;
     const PairConst k(p);
 
@@ -449,7 +428,7 @@ pair_kernel(const T* __restrict__ gin, T* __restrict__ gout, const __grid_consta
         if (inner) {
             const T* row = cin + (long long)(rr - 1) * p.rs;
 #pragma unroll
-            for (int a = 0; a < 9; a++) v[a].load(row + q.kin[a]);   // one multiply-add a population
+            for (int a = 0; a < 9; a++) v[a].load(row + kin[a]);   // one multiply-add a population
         } else {
 #pragma unroll
             for (int a = 0; a < 9; a++) {
@@ -473,7 +452,7 @@ pair_kernel(const T* __restrict__ gin, T* __restrict__ gout, const __grid_consta
                 v[a].scalars(t);
             }
         }
-        const int band = srow != nullptr ? __ldg(srow + rr * q.nstrip) : -1;
+        const int band = srow != nullptr ? __ldg(srow + rr * nstrip) : -1;
         P2 f[9][NP];
 #pragma unroll
         for (int a = 0; a < 9; a++) {
@@ -489,7 +468,7 @@ pair_kernel(const T* __restrict__ gin, T* __restrict__ gout, const __grid_consta
         if (uniform_force || band >= 0) {
             if (band >= 0) {
                 cudaGridDependencySynchronize();
-                pair_spread<NPL>(q.fb1, band, lane, Fx, Fy);
+                pair_spread<NPL>(fb1, band, lane, Fx, Fy);
             }
             collide_pairs<true, NP>(f, p, k, Fx, Fy, Raw<T>::kScale);
         } else {
@@ -508,7 +487,7 @@ pair_kernel(const T* __restrict__ gin, T* __restrict__ gout, const __grid_consta
     for (int j = warp; j < TH; j += NW) {
         const int y = y0 + j;
         if (y >= ny) break;
-        const int band = srow != nullptr ? __ldg(srow + y * q.nstrip) : -1;
+        const int band = srow != nullptr ? __ldg(srow + y * nstrip) : -1;
         const T* const trow = tile + (j + 1) * C::W + NPL * lane;
         const bool inner = pery || (y > 0 && y < ny - 1);
         P2 f[9][NP];
@@ -539,7 +518,7 @@ pair_kernel(const T* __restrict__ gin, T* __restrict__ gout, const __grid_consta
         T* const row = cout + (long long)y * p.rs;
         P2 Fx[NP] = {}, Fy[NP] = {};
         if (uniform_force || band >= 0) {
-            if (band >= 0) pair_spread<NPL>(q.fb2, band, lane, Fx, Fy);
+            if (band >= 0) pair_spread<NPL>(fb2, band, lane, Fx, Fy);
             collide_pairs<true, NP>(f, p, k, Fx, Fy, Raw<T>::kScale);
         } else {
             collide_pairs<false, NP>(f, p, k, Fx, Fy, Raw<T>::kScale);
@@ -556,24 +535,97 @@ pair_kernel(const T* __restrict__ gin, T* __restrict__ gout, const __grid_consta
     }
 }
 
+// Last of the reduction blocks: the step counter.
+__device__ __forceinline__ void pair_finish(unsigned long long* counter, unsigned long long step, unsigned* done,
+                                            int nred) {
+    __syncthreads();
+    if (threadIdx.x == 0 && counter != nullptr) {
+        __threadfence();
+        if (atomicAdd(done, 1u) == (unsigned)nred - 1u) {
+            *counter = step + 2ull;
+            *done = 0u;
+        }
+    }
+}
+
+template <typename T, int NPL, int NW, int TH, int MINB>
+__global__ void __launch_bounds__(32 * NW, MINB)
+pair_kernel(const T* __restrict__ gin, T* __restrict__ gout, const __grid_constant__ LatticeParams p,
+            const __grid_constant__ PairForces q, int nred) {
+    cudaTriggerProgrammaticLaunchCompletion();
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    // The first nred blocks reduce the body forces of both steps while the
+    // others work; the last of them to finish advances the step counter.
+    if ((int)blockIdx.x < nred) {
+        if (p.nbody > 0) cudaGridDependencySynchronize();
+        const unsigned long long step = p.step != nullptr ? *p.step : 0ull;
+        const int half = NW / 2, w = (int)threadIdx.x >> 5;
+        if (w < half) body_forces(p, q.F1, step, blockIdx.x * half + w, nred * half);
+        else if (w < 2 * half) body_forces(p, p.F, step + 1ull, blockIdx.x * half + w - half, nred * half);
+        pair_finish(p.step, step, q.done, nred);
+        return;
+    }
+    const int b = (int)blockIdx.x - nred;
+    const int c = b / q.nstrip, s = b - c * q.nstrip;
+    pair_tile<T, NPL, NW, TH>(gin, gout, p, q.kin, q.strip_row, q.nstrip, q.fb1, q.fb2, s, c * TH,
+                              reinterpret_cast<T*>(smem_raw));
+}
+
+// Batched form: the tiles of all lattices in one launch; a block copies its
+// lattice's description to shared memory first.
+template <typename T, int NPL, int NW, int TH, int MINB>
+__global__ void __launch_bounds__(32 * NW, MINB)
+pair_batch_kernel(const T* __restrict__ gin, T* __restrict__ gout, const __grid_constant__ PairBatch b,
+                  const __grid_constant__ PairForces q, int nred) {
+    cudaTriggerProgrammaticLaunchCompletion();
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    if ((int)blockIdx.x < nred) {
+        if (b.nbody > 0) cudaGridDependencySynchronize();
+        const unsigned long long step = *b.step;
+        const int half = NW / 2, w = (int)threadIdx.x >> 5;
+        if (w < half)
+            body_forces(b.nbody, b.body_rng, 2, b.body_scale, b.hist, b.hist_len, q.F1, step, blockIdx.x * half + w,
+                        nred * half);
+        else if (w < 2 * half)
+            body_forces(b.nbody, b.body_rng, 2, b.body_scale, b.hist, b.hist_len, b.F2, step + 1ull,
+                        blockIdx.x * half + w - half, nred * half);
+        pair_finish(b.step, step, q.done, nred);
+        return;
+    }
+    __shared__ __align__(16) LatticeParams sp;
+    __shared__ __align__(16) PairLattice sl;
+    const int4 t = __ldg(b.tile + ((int)blockIdx.x - nred));
+    {
+        const int* a = reinterpret_cast<const int*>(b.descs + t.x);
+        const int* c = reinterpret_cast<const int*>(b.lat + t.x);
+        for (int i = threadIdx.x; i < (int)(sizeof(LatticeParams) / 4); i += 32 * NW)
+            reinterpret_cast<int*>(&sp)[i] = __ldg(a + i);
+        for (int i = threadIdx.x; i < (int)(sizeof(PairLattice) / 4); i += 32 * NW)
+            reinterpret_cast<int*>(&sl)[i] = __ldg(c + i);
+    }
+    __syncthreads();
+    pair_tile<T, NPL, NW, TH>(gin + sl.off, gout + sl.off, sp, sl.kin, sl.strip_row, sl.nstrip, q.fb1, q.fb2, t.y, t.z,
+                              reinterpret_cast<T*>(smem_raw));
+}
+
 // Spread (Eq. 15) of the forces F, one thread per band node of a strip that has
 // terms: nodes[t] = (slot in fb, first term, end of terms).
-__device__ __forceinline__ void spread_node(const LatticeParams& p, const float2* F, const PairForces& q, float* fb,
+__device__ __forceinline__ void spread_node(const CsrEntry* csr, const float2* F, const PairForces& q, float* fb,
                                             int t) {
     if (t >= q.nnode) return;
     const int4 n = __ldg(q.nodes + t);
     float fx, fy;
-    spread_terms(p, F, n.y, n.z, fx, fy);
+    spread_terms(csr, F, n.y, n.z, fx, fy);
     fb[n.x] = fx;
     fb[n.x + 32 * q.npl] = fy;
 }
 
-__global__ void __launch_bounds__(128) spread_kernel(LatticeParams p, PairForces q) {
+__global__ void __launch_bounds__(128) spread_kernel(const CsrEntry* csr, const float2* F, PairForces q) {
     // Its dependent may start at once: this grid starts after ib_force's wait for
     // the previous pair (ib_pair_kernel launches it the same way).
     cudaTriggerProgrammaticLaunchCompletion();
     cudaGridDependencySynchronize();
-    spread_node(p, p.F, q, q.fb2, (int)(blockIdx.x * blockDim.x + threadIdx.x));
+    spread_node(csr, F, q, q.fb2, (int)(blockIdx.x * blockDim.x + threadIdx.x));
 }
 
 // Forces of the second step, one warp per marker.  The lanes redo the first
@@ -585,23 +637,10 @@ __global__ void __launch_bounds__(128) spread_kernel(LatticeParams p, PairForces
 constexpr int kIbPairThreads = 128;
 
 template <typename T, int S>
-__global__ void __launch_bounds__(kIbPairThreads)
-ib_pair_kernel(const T* __restrict__ g, LatticeParams p, IbParams q, PairForces r, int mblocks) {
-    constexpr int P = S + 2, W = kIbPairThreads / 32;
-    __shared__ float patch[W][9][P * P];
-    const float2* const F1 = r.F1;
-    // ib_force, whose dependent this is, has waited for the previous pair of
-    // steps before letting this grid start, so everything after it may start too:
-    // the pair kernel's warps off the band need nothing else.
-    cudaTriggerProgrammaticLaunchCompletion();
-    if ((int)blockIdx.x >= mblocks) {   // the first step's spread
-        cudaGridDependencySynchronize();
-        spread_node(p, F1, r, r.fb1, ((int)blockIdx.x - mblocks) * kIbPairThreads + (int)threadIdx.x);
-        return;
-    }
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const long long m = (long long)blockIdx.x * W + warp;
-    if (m >= q.nmark) return;   // whole warps
+__device__ __forceinline__ void ib_pair_marker(const T* __restrict__ g, const LatticeParams& p, const IbParams& q,
+                                               const float2* F1, long long m, float (*patch)[(S + 2) * (S + 2)]) {
+    constexpr int P = S + 2;
+    const int lane = threadIdx.x & 31;
     const Marker* mk = q.mk + m;
     const MarkerAux ax = q.aux[m];
     const int xa = __ldg(&mk->xs[0]), ya = __ldg(&mk->ys[0]);
@@ -633,13 +672,13 @@ ib_pair_kernel(const T* __restrict__ g, LatticeParams p, IbParams q, PairForces 
         const int seg = __ldg(p.seg_index + y * p.nseg + x / kSeg);
         if (seg >= 0) {
             const int* ptr = p.seg_ptr + (long long)seg * (kSeg + 1) + (x % kSeg);
-            spread_terms(p, F1, __ldg(ptr), __ldg(ptr + 1), Fx[0], Fy[0]);
+            spread_terms(p.csr, F1, __ldg(ptr), __ldg(ptr + 1), Fx[0], Fy[0]);
         }
         const bool forced = seg >= 0 || p.gx != 0.f || p.gy != 0.f;
         collide_nodes<T, 1>(f, p, Fx, Fy, forced, [&](int a, const float (&o)[1]) {
             T st;
             Raw<T>::template stv<1>(&st, o);
-            patch[warp][a][e] = Io<T>::ld1s(&st);
+            patch[a][e] = Io<T>::ld1s(&st);
         });
     }
     __syncwarp();
@@ -656,7 +695,7 @@ ib_pair_kernel(const T* __restrict__ g, LatticeParams p, IbParams q, PairForces 
             y_source(a, y, p, pa, sy, dx, add);
             const bool wall = p.bcy != kBcyPeriodic && y - ey(a) != sy;
             const int row = wall ? sj + 1 : sj + 1 - ey(a);
-            d[a] = patch[warp][pa][row * P + si + 1 + dx] + add;
+            d[a] = patch[pa][row * P + si + 1 + dx] + add;
         }
         const Moments mo = moments(d, p.urx, p.ury);
         wr = w * mo.drho;
@@ -679,6 +718,47 @@ ib_pair_kernel(const T* __restrict__ g, LatticeParams p, IbParams q, PairForces 
         q.rhol[m] = rl;
         if (!(rl > 0.f) || !isfinite(dFx) || !isfinite(dFy)) atomicOr(q.status, kStatusUnstable);
     }
+}
+
+template <typename T, int S>
+__global__ void __launch_bounds__(kIbPairThreads)
+ib_pair_kernel(const T* __restrict__ g, LatticeParams p, IbParams q, PairForces r, int mblocks) {
+    constexpr int W = kIbPairThreads / 32;
+    __shared__ float patch[W][9][(S + 2) * (S + 2)];
+    // ib_force, whose dependent this is, has waited for the previous pair of
+    // steps before letting this grid start, so everything after it may start too:
+    // the pair kernel's warps off the band need nothing else.
+    cudaTriggerProgrammaticLaunchCompletion();
+    if ((int)blockIdx.x >= mblocks) {   // the first step's spread
+        cudaGridDependencySynchronize();
+        spread_node(p.csr, r.F1, r, r.fb1, ((int)blockIdx.x - mblocks) * kIbPairThreads + (int)threadIdx.x);
+        return;
+    }
+    const int warp = threadIdx.x >> 5;
+    const long long m = (long long)blockIdx.x * W + warp;
+    if (m >= q.nmark) return;   // whole warps
+    ib_pair_marker<T, S>(g, p, q, r.F1, m, patch[warp]);
+}
+
+// Batched form: MarkerAux.body holds the marker's lattice.
+template <typename T, int S>
+__global__ void __launch_bounds__(kIbPairThreads)
+ib_pair_batch_kernel(const T* __restrict__ g, const LatticeParams* __restrict__ descs,
+                     const unsigned long long* __restrict__ case_off, IbParams q, PairForces r,
+                     const CsrEntry* csr, int mblocks) {
+    constexpr int W = kIbPairThreads / 32;
+    __shared__ float patch[W][9][(S + 2) * (S + 2)];
+    cudaTriggerProgrammaticLaunchCompletion();   // as in ib_pair_kernel
+    if ((int)blockIdx.x >= mblocks) {
+        cudaGridDependencySynchronize();
+        spread_node(csr, r.F1, r, r.fb1, ((int)blockIdx.x - mblocks) * kIbPairThreads + (int)threadIdx.x);
+        return;
+    }
+    const int warp = threadIdx.x >> 5;
+    const long long m = (long long)blockIdx.x * W + warp;
+    if (m >= q.nmark) return;
+    const int c = q.aux[m].body;
+    ib_pair_marker<T, S>(g + case_off[c], descs[c], q, r.F1, m, patch[warp]);
 }
 
 cudaLaunchConfig_t config(unsigned grid, unsigned threads, bool pdl, cudaLaunchAttribute* attr, cudaStream_t st) {
@@ -737,7 +817,7 @@ int pair_npl(int storage, int bcx, int nx, int ny) {
     if (storage != kStoreF32 || (long long)nx * ny >= (1ll << 22)) return 4;
     return bcx == kBcxInout && (nx - 1) % pair_own(2) == 0 ? 4 : 2;
 }
-int pair_strips(const LatticeParams& p, int npl) { return (p.nx + pair_own(npl) - 1) / pair_own(npl); }
+int pair_tile_rows(int npl) { return npl == 2 ? 6 : 7; }
 
 namespace {
 
@@ -747,7 +827,72 @@ cudaError_t pair_t(const void* gin, void* gout, const LatticeParams& p, const Pa
     return pair_tn<T, 4, 9, 7, 3>(gin, gout, p, q, pdl, st);
 }
 
+template <typename T, int NPL, int NW, int TH, int MINB>
+cudaError_t pair_batch_tn(const void* gin, void* gout, const PairBatch& b, const PairForces& q, bool pdl,
+                          cudaStream_t st) {
+    using C = PairTile<T, NPL, TH>;
+    auto kern = pair_batch_kernel<T, NPL, NW, TH, MINB>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::kShared);
+    if (e != cudaSuccess) return e;
+    const int nred = std::min(16, std::max(1, (b.nbody + 2 * NW - 1) / (2 * NW)));
+    cudaLaunchAttribute attr[1];
+    cudaLaunchConfig_t cfg = config((unsigned)(b.ntile + nred), 32 * NW, pdl, attr, st);
+    cfg.dynamicSmemBytes = C::kShared;
+    return cudaLaunchKernelEx(&cfg, kern, (const T*)gin, (T*)gout, b, q, nred);
+}
+
+template <typename T>
+cudaError_t pair_batch_t(const void* gin, void* gout, const PairBatch& b, const PairForces& q, bool pdl,
+                         cudaStream_t st) {
+    if (q.npl == 2) return pair_batch_tn<T, 2, 8, 6, 5>(gin, gout, b, q, pdl, st);
+    return pair_batch_tn<T, 4, 9, 7, 3>(gin, gout, b, q, pdl, st);
+}
+
+template <typename T>
+cudaError_t ib_pair_batch_t(int width, const void* g, const LatticeParams* descs, const unsigned long long* off,
+                            const IbParams& q, const PairForces& r, const CsrEntry* csr, bool pdl, cudaStream_t st) {
+    constexpr int W = kIbPairThreads / 32;
+    const int mb = (q.nmark + W - 1) / W;
+    cudaLaunchAttribute attr[1];
+    const cudaLaunchConfig_t cfg =
+        config((unsigned)(mb + (r.nnode + kIbPairThreads - 1) / kIbPairThreads), kIbPairThreads, pdl, attr, st);
+    switch (width) {
+    case 2: return cudaLaunchKernelEx(&cfg, ib_pair_batch_kernel<T, 2>, (const T*)g, descs, off, q, r, csr, mb);
+    case 3: return cudaLaunchKernelEx(&cfg, ib_pair_batch_kernel<T, 3>, (const T*)g, descs, off, q, r, csr, mb);
+    case 4: return cudaLaunchKernelEx(&cfg, ib_pair_batch_kernel<T, 4>, (const T*)g, descs, off, q, r, csr, mb);
+    default: return cudaErrorInvalidValue;
+    }
+}
+
+cudaError_t spread_second(const CsrEntry* csr, const float2* F, const PairForces& r, bool pdl, cudaStream_t st) {
+    cudaLaunchAttribute attr[1];
+    const cudaLaunchConfig_t cfg = config((unsigned)((r.nnode + 127) / 128), 128, pdl, attr, st);
+    return cudaLaunchKernelEx(&cfg, spread_kernel, csr, F, r);
+}
+
 }  // namespace
+
+cudaError_t launch_pair_batch(int storage, const void* gin, void* gout, const PairBatch& b, const PairForces& q,
+                              bool pdl, cudaStream_t st) {
+    switch (storage) {
+    case kStoreF32: return pair_batch_t<float>(gin, gout, b, q, pdl, st);
+    case kStoreF16: return pair_batch_t<__half>(gin, gout, b, q, pdl, st);
+    case kStoreBF16: return pair_batch_t<__nv_bfloat16>(gin, gout, b, q, pdl, st);
+    default: return cudaErrorInvalidValue;
+    }
+}
+
+cudaError_t launch_ib_pair_batch(int storage, int width, const void* g, const LatticeParams* descs,
+                                 const unsigned long long* case_off, const IbParams& q, const PairForces& r,
+                                 const CsrEntry* csr, bool pdl, cudaStream_t st) {
+    cudaError_t e = cudaErrorInvalidValue;
+    switch (storage) {
+    case kStoreF32: e = ib_pair_batch_t<float>(width, g, descs, case_off, q, r, csr, pdl, st); break;
+    case kStoreF16: e = ib_pair_batch_t<__half>(width, g, descs, case_off, q, r, csr, pdl, st); break;
+    case kStoreBF16: e = ib_pair_batch_t<__nv_bfloat16>(width, g, descs, case_off, q, r, csr, pdl, st); break;
+    }
+    return e != cudaSuccess ? e : spread_second(csr, q.F_out, r, pdl, st);
+}
 
 cudaError_t launch_pair(int storage, const void* gin, void* gout, const LatticeParams& p, const PairForces& q, bool pdl,
                         cudaStream_t st) {
@@ -767,10 +912,7 @@ cudaError_t launch_ib_pair(int storage, int width, const void* g, const LatticeP
     case kStoreF16: e = ib_pair_t<__half>(width, g, p, q, r, pdl, st); break;
     case kStoreBF16: e = ib_pair_t<__nv_bfloat16>(width, g, p, q, r, pdl, st); break;
     }
-    if (e != cudaSuccess) return e;
-    cudaLaunchAttribute attr[1];
-    const cudaLaunchConfig_t cfg = config((unsigned)((r.nnode + 127) / 128), 128, pdl, attr, st);
-    return cudaLaunchKernelEx(&cfg, spread_kernel, p, r);
+    return e != cudaSuccess ? e : spread_second(p.csr, q.F_out, r, pdl, st);
 }
 
 }  // namespace btdf

@@ -171,4 +171,35 @@ void build_marker_tables(int nx, int ny, int nseg, int delta, int width, bool px
     }
 }
 
+// The band as the pair kernel's strips see it (PairForces), from the spreading
+// table: each strip with the columns beside it, so a node near a border belongs
+// to two strips (and, wrapped, a narrow periodic lattice's node to several).
+// Appends; rows are numbered from nsrow, terms from term0.
+void build_pair_tables(int nx, int ny, int nseg, bool px, int npl, int nstrip, const std::vector<int>& keys,
+                       const std::vector<int>& seg_ptr, int term0, std::vector<int>& strip_row,
+                       std::vector<int4>& nodes, int& nsrow) {
+    const int own = pair_own(npl);
+    const size_t r0 = strip_row.size();
+    strip_row.resize(r0 + (size_t)ny * nstrip, -1);
+    nodes.reserve(nodes.size() + keys.size() * 16);
+    for (size_t s = 0; s < keys.size(); s++) {
+        const int y = keys[s] / nseg, xs = keys[s] % nseg * kSeg;
+        int* const rows = &strip_row[r0 + (size_t)y * nstrip];
+        const int* const ptr = &seg_ptr[s * (kSeg + 1)];
+        for (int i = 0; i < kSeg; i++) {
+            if (ptr[i + 1] <= ptr[i]) continue;
+            for (int x = px ? xs + i - nx : xs + i; x < nstrip * own + npl; x += nx) {
+                for (int k = std::max(0, (x - npl) / own); k < nstrip; k++) {
+                    const int c = x - (k * own - npl);
+                    if (c < 0) break;
+                    if (c >= 32 * npl) continue;
+                    if (rows[k] < 0) rows[k] = nsrow++;
+                    nodes.push_back(make_int4(rows[k] * 64 * npl + c, term0 + ptr[i], term0 + ptr[i + 1], 0));
+                }
+                if (!px) break;
+            }
+        }
+    }
+}
+
 }  // namespace btdf

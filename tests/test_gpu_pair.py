@@ -103,3 +103,28 @@ def test_many_inlet_and_outlet_nodes(storage):
     # roundings of the row ends that differ once in thousands of nodes
     for bcx in (W.BCX_INOUT, W.BCX_CONVECTIVE):
         compare(case(90, 4001, bcx, W.BCY_FREESLIP, tau=0.53, bodies=[(45.0, 2000.0, 9.0)]), storage, steps=(1, 130))
+
+
+@pytest.mark.parametrize("storage", STORAGES)
+def test_batch_pairs(storage):
+    """The batch's pairs (automatic shape) against launch shape 1, which steps
+    singly: lattices of both strip widths' edges, every boundary kind, with and
+    without bodies."""
+    cases = [case(nx, ny, bcx, bcy, bodies=bodies, gx=1e-6 if bcx == W.BCX_PERIODIC else 0.0)
+             for nx, ny, bcx, bcy, bodies in [
+                 (121, 37, W.BCX_INOUT, W.BCY_FREESLIP, [(100.0, 18.4, 9.0), (15.2, 20.1, 7.0)]),
+                 (64, 29, W.BCX_PERIODIC, W.BCY_PERIODIC, [(0.3, 12.0, 6.0)]),
+                 (119, 30, W.BCX_PERIODIC, W.BCY_NOSLIP, [(40.0, 15.0, 8.0)]),
+                 (48, 36, W.BCX_INOUT, W.BCY_NOSLIP, []),
+                 (250, 64, W.BCX_INOUT, W.BCY_PERIODIC, [(120.3, 30.0, 12.0)])]]
+    a = B.Batch.from_cases(cases, storage=storage, history_len=16)
+    b = B.Batch.from_cases(cases, storage=storage, history_len=16)
+    b.tune(1)
+    for n in (1, 2, 5, 66):
+        a.step(n)
+        b.step(n)
+        for i in range(len(cases)):
+            assert np.array_equal(a.field(i, B.FIELD_POPS), b.field(i, B.FIELD_POPS)), (n, i)
+        for k in range(len(a.bodies)):
+            fa, fb = (x.forces(k, x.steps - min(n, 8), min(n, 8)) for x in (a, b))
+            assert np.array_equal(fa[0], fb[0]) and np.array_equal(fa[1], fb[1]), (n, k)
