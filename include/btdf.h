@@ -264,9 +264,8 @@ int btdf_profile_read(btdf_ctx *ctx, double *ms_ib, double *ms_lbm, int64_t *lau
 
 /* Variant of the fused collide-stream kernel.  Results do not depend on it.
  *   0 automatic: two steps per pass over the lattice where the call's steps come
- *     in pairs and that is the faster form (nf = 1, no box, every marker support
- *     inside the lattice and off the inlet and outlet columns; FP32 storage with
- *     bodies: from 2^17 nodes up); single steps otherwise: on lattices of at least 2^23 nodes 11 for FP32 and 12 for
+ *     in pairs (nf = 1, no box, every marker support inside the lattice and off
+ *     the inlet and outlet columns); single steps otherwise: on lattices of at least 2^23 nodes 11 for FP32 and 12 for
  *     FP16 / BF16 storage (11 where no tensor maps could be encoded), on
  *     smaller ones 2 for FP32 and 11 for FP16 / BF16 (the autotuner's usual
  *     picks on a GB300)

@@ -508,16 +508,14 @@ bool pairs_possible(const btdf_ctx* ctx) {
     return !ctx->prof && !ctx->d_box && (ctx->nmark == 0 || (ctx->cfg.nf == 1 && ctx->markers_inside));
 }
 
-// Whether the context takes them: with the automatic variant where they are the
-// faster form, or after the autotuner found them so.  With bodies a pair's chain
-// of four launches takes about 12 us; two single steps of a small FP32 lattice
-// take as long (160 x 80: 12.2 against 12.7 us; 800 x 400: 14.5 against 14.3;
-// 1200 x 600: 19.0 against 15.2), the slower 16-bit steps do not (160 x 80: 17.4
-// against 12.7).  Without bodies there is no chain (160 x 80: 7.6 against 4.0).
+// Whether the context takes them: with the automatic variant (they are the faster
+// form at every size: us a step, singly -> in pairs, with one body: 160 x 80 FP32
+// 6.1 -> 4.9, FP16 8.7 -> 5.6; 800 x 400 7.2 -> 5.9 and 8.4 -> 6.2; 1600 x 800
+// 14.8 -> 11.6 and 13.3 -> 11.1; 160 x 80 without bodies 3.8 -> 2.0), or after the
+// autotuner found them so.
 bool pairs_allowed(const btdf_ctx* ctx) {
     if (!pairs_possible(ctx)) return false;
-    if (ctx->variant != kVarAuto || ctx->grid_override != 0) return ctx->pairs_tuned;
-    return ctx->nmark == 0 || ctx->cfg.storage != kStoreF32 || (long long)ctx->cfg.nx * ctx->cfg.ny >= (1ll << 17);
+    return ctx->variant == kVarAuto && ctx->grid_override == 0 ? true : ctx->pairs_tuned;
 }
 
 // Tables of the pair kernels for the current markers.

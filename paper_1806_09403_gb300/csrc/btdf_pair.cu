@@ -7,8 +7,9 @@
 // second step needs the first step's result on its eight neighbours only.
 // pair_kernel keeps that result in shared memory, so a pair of steps moves what a
 // single one moves.  Measured, us a step, single -> pair: 8192 x 4096 with 400
-// bodies FP32 343 -> 234, FP16 220 -> 208; 1600 x 800 with one body FP32
-// 14.8 -> 11.5, FP16 13.3 -> 11.1; 1601 x 1601 BF16 28.2 -> 20.
+// bodies FP32 343 -> 232, FP16 220 -> 209; 1600 x 800 with one body FP32
+// 14.8 -> 11.6, FP16 13.3 -> 11.1; 1601 x 1601 BF16 28.2 -> 21.7; 128 lattices in
+// a batch FP32 395 -> 242.
 //
 // The marker forces of the second step are needed before the pass that would
 // produce the state they are interpolated from.  ib_pair_kernel redoes the
@@ -20,7 +21,10 @@
 // (those of the second, and the first step's spread over the band nodes),
 // spread (the second step's), pair (both collisions, streamings and force
 // histories).  Each is a programmatic dependent of the one before; tiles of the
-// pair kernel off the band wait for none of them.
+// pair kernel off the band wait for none of them.  What is on the chain's path is
+// kept short: the kernels after ib_force have loaded everything but the forces
+// (state, tables, the first terms of every spread) before they wait.  With those
+// loads after the wait, entry by entry, a pair on 160 x 80 took 12.7 us, now 9.8.
 #include "btdf_internal.cuh"
 #include "btdf_device.cuh"
 #include "btdf_collide.cuh"
@@ -279,18 +283,42 @@ template <int NPL> struct Vec<float, NPL> {
     }
 };
 
-// Spread force (Eq. 15) of the terms b .. e-1.
-__device__ __forceinline__ void spread_terms(const CsrEntry* csr, const float2* F, int b, int e, float& sx,
-                                             float& sy) {
-    sx = 0.f;
-    sy = 0.f;
-    for (int k = b; k < e; k++) {
-        const CsrEntry c = csr[k];
-        const float2 f = F[c.marker];
-        sx = __fmaf_rn(c.w, f.x, sx);
-        sy = __fmaf_rn(c.w, f.y, sy);
+// Spread force (Eq. 15) of the terms b .. e-1.  The first kTerms of them are
+// loaded ahead (no kernel of a step writes them), so that only the loads of the
+// forces, all at once, follow the wait for the kernel that writes those.
+constexpr int kTerms = 8;
+struct SpreadTerms {
+    CsrEntry c[kTerms];
+    int b, e;
+    __device__ __forceinline__ void load(const CsrEntry* csr, int b_, int e_) {
+        b = b_;
+        e = e_;
+#pragma unroll
+        for (int k = 0; k < kTerms; k++) {
+            c[k] = CsrEntry{0, 0.f};
+            if (b + k < e) c[k] = csr[b + k];
+        }
     }
-}
+    __device__ __forceinline__ void sum(const CsrEntry* csr, const float2* F, float& sx, float& sy) const {
+        float2 f[kTerms];
+#pragma unroll
+        for (int k = 0; k < kTerms; k++) f[k] = b + k < e ? F[c[k].marker] : make_float2(0.f, 0.f);
+        sx = 0.f;
+        sy = 0.f;
+#pragma unroll
+        for (int k = 0; k < kTerms; k++)
+            if (b + k < e) {
+                sx = __fmaf_rn(c[k].w, f[k].x, sx);
+                sy = __fmaf_rn(c[k].w, f[k].y, sy);
+            }
+        for (int k = b + kTerms; k < e; k++) {
+            const CsrEntry t = csr[k];
+            const float2 v = F[t.marker];
+            sx = __fmaf_rn(t.w, v.x, sx);
+            sy = __fmaf_rn(t.w, v.y, sy);
+        }
+    }
+};
 
 // A tile of 30 * NPL columns x TH rows per block.  First step: the block's warps
 // pull the TH + 2 rows of 32 * NPL columns around the tile from memory, collide
@@ -299,14 +327,14 @@ __device__ __forceinline__ void spread_terms(const CsrEntry* csr, const float2* 
 // warp takes a row at a time, NPL consecutive nodes per lane; the outer two lanes
 // hold the columns beside the tile.
 //
-// What bounds it: instructions.  On 4096 x 2048 FP32 it moves 560 MB a pair at
-// 4.5 TB/s (0.67 of the measured copy rate) with the issue slots 65% busy at 27
-// warps an SM, FP16 half the bytes in nearly the same time with them 72% busy and
-// the FMA pipe throttling; FP32 arithmetic is 77 of about 300 instructions per
-// row of 64 nodes and step.  Small tiles, although their halo costs 14-20% more
-// node updates, keep the register count low and 3 to 5 blocks an SM resident, so
-// that one block's barrier and loads hide behind the others: tiles of 14 rows
-// with two blocks an SM took 265 (FP32) and 249 us (FP16) a step on 8192 x 4096.
+// What bounds it: instructions.  On 8192 x 4096 FP32 it moves 2.42 GB a pair at
+// 5.2 TB/s (0.78 of the measured copy rate), FP16 half the bytes in nearly the same
+// time; on 4096 x 2048 the issue slots are 65% (FP32) and 72% (FP16) busy, with the
+// FMA pipe throttling; FP32 arithmetic is 77 of about 300 instructions per row of
+// 64 nodes and step.  Small tiles, although their halo costs 14-20% more node
+// updates, keep the register count low and 3 to 5 blocks an SM resident, so that one block's
+// barrier and loads hide behind the others: tiles of 14 rows with two blocks an SM
+// took 235 to 265 us a step on 8192 x 4096.
 // A form that walks down the rows with the first step's rows in registers
 // (128-168 registers, 3-4 warps a scheduler) stayed at 245-255 us there and made
 // a chain of a small lattice's rows (14.4 us at 1600 x 800).
@@ -322,6 +350,8 @@ struct PairTile {
 // lane below's last (old: the convective outlet's previous column; keep: write
 // the new one).  Inner nodes take the wall's constant with one rounding, row
 // ends (g; those of a periodic lattice too) with two, as the single steps do.
+// One population at a time: arrays of the lane's nodes would raise the register
+// count of the whole kernel.
 template <typename T, int NPL>
 __device__ __forceinline__ void pair_boundaries(P2 (&fp)[9][NPL / 2], const LatticeParams& p, int x0, int y, bool ends,
                                                 const float* old, bool keep) {
@@ -612,10 +642,14 @@ pair_batch_kernel(const T* __restrict__ gin, T* __restrict__ gout, const __grid_
 // terms: nodes[t] = (slot in fb, first term, end of terms).
 __device__ __forceinline__ void spread_node(const CsrEntry* csr, const float2* F, const PairForces& q, float* fb,
                                             int t) {
+    int4 n = make_int4(0, 0, 0, 0);
+    SpreadTerms terms;
+    if (t < q.nnode) n = __ldg(q.nodes + t);
+    terms.load(csr, n.y, n.z);
+    cudaGridDependencySynchronize();
     if (t >= q.nnode) return;
-    const int4 n = __ldg(q.nodes + t);
     float fx, fy;
-    spread_terms(csr, F, n.y, n.z, fx, fy);
+    terms.sum(csr, F, fx, fy);
     fb[n.x] = fx;
     fb[n.x + 32 * q.npl] = fy;
 }
@@ -624,7 +658,6 @@ __global__ void __launch_bounds__(128) spread_kernel(const CsrEntry* csr, const 
     // Its dependent may start at once: this grid starts after ib_force's wait for
     // the previous pair (ib_pair_kernel launches it the same way).
     cudaTriggerProgrammaticLaunchCompletion();
-    cudaGridDependencySynchronize();
     spread_node(csr, F, q, q.fb2, (int)(blockIdx.x * blockDim.x + threadIdx.x));
 }
 
@@ -646,19 +679,28 @@ __device__ __forceinline__ void ib_pair_marker(const T* __restrict__ g, const La
     const int xa = __ldg(&mk->xs[0]), ya = __ldg(&mk->ys[0]);
     const bool act = lane < S * S;
     const float w = act ? __ldg(&mk->w[lane]) : 0.f;
-    cudaGridDependencySynchronize();
+    // Everything but the forces F1 is there before ib_force has finished: the
+    // state g (ib_force let this grid start after its wait for it) and the tables.
+    constexpr int R = (P * P + 31) / 32;
+    float f[R][9][1];
+    SpreadTerms terms[R];
+    bool valid[R], band[R];
 #pragma unroll
-    for (int e = lane; e < P * P; e += 32) {
+    for (int k = 0; k < R; k++) {
+        const int e = lane + 32 * k;
         const int j = e / P, i = e - j * P;
         // support columns are consecutive up to a periodic wrap
         int x = xa + i - 1, y = ya + j - 1;
         if (p.bcx == kBcxPeriodic) x = ((x % p.nx) + p.nx) % p.nx;
         if (p.bcy == kBcyPeriodic) y = ((y % p.ny) + p.ny) % p.ny;
-        if (x < 0 || x >= p.nx || y < 0 || y >= p.ny) continue;
-        float d[9], f[9][1], Fx[1] = {0.f}, Fy[1] = {0.f};
+        valid[k] = e < P * P && x >= 0 && x < p.nx && y >= 0 && y < p.ny;
+        band[k] = false;
+        terms[k].load(p.csr, 0, 0);
+        if (!valid[k]) continue;
+        float d[9];
         gather_node<T>(g, p, true, x, y, d);
 #pragma unroll
-        for (int a = 0; a < 9; a++) f[a][0] = d[a] * Raw<T>::kScale;
+        for (int a = 0; a < 9; a++) f[k][a][0] = d[a] * Raw<T>::kScale;
         // the LBM kernels add a bounce-back wall's constant with one rounding
         // on inner columns
         if (p.bcy == kBcyNoslip && (y == 0 || y == p.ny - 1) && x > 0 && x < p.nx - 1) {
@@ -666,16 +708,25 @@ __device__ __forceinline__ void ib_pair_marker(const T* __restrict__ g, const La
             for (int a = 0; a < 9; a++)
                 if ((ey(a) > 0 && y == 0) || (ey(a) < 0 && y == p.ny - 1)) {
                     const float v = Io<T>::ld1(g + p.poff[opposite(a)] + (unsigned)y * p.rs + (unsigned)x);
-                    f[a][0] = __fmaf_rn(-6.0f * wt(a), p.eur[a], v) * Raw<T>::kScale;
+                    f[k][a][0] = __fmaf_rn(-6.0f * wt(a), p.eur[a], v) * Raw<T>::kScale;
                 }
         }
         const int seg = __ldg(p.seg_index + y * p.nseg + x / kSeg);
         if (seg >= 0) {
             const int* ptr = p.seg_ptr + (long long)seg * (kSeg + 1) + (x % kSeg);
-            spread_terms(p.csr, F1, __ldg(ptr), __ldg(ptr + 1), Fx[0], Fy[0]);
+            terms[k].load(p.csr, __ldg(ptr), __ldg(ptr + 1));
+            band[k] = true;
         }
-        const bool forced = seg >= 0 || p.gx != 0.f || p.gy != 0.f;
-        collide_nodes<T, 1>(f, p, Fx, Fy, forced, [&](int a, const float (&o)[1]) {
+    }
+    cudaGridDependencySynchronize();
+#pragma unroll
+    for (int k = 0; k < R; k++) {
+        if (!valid[k]) continue;
+        const int e = lane + 32 * k;
+        float Fx[1], Fy[1];
+        terms[k].sum(p.csr, F1, Fx[0], Fy[0]);
+        const bool forced = band[k] || p.gx != 0.f || p.gy != 0.f;
+        collide_nodes<T, 1>(f[k], p, Fx, Fy, forced, [&](int a, const float (&o)[1]) {
             T st;
             Raw<T>::template stv<1>(&st, o);
             patch[a][e] = Io<T>::ld1s(&st);
@@ -730,7 +781,6 @@ ib_pair_kernel(const T* __restrict__ g, LatticeParams p, IbParams q, PairForces 
     // the pair kernel's warps off the band need nothing else.
     cudaTriggerProgrammaticLaunchCompletion();
     if ((int)blockIdx.x >= mblocks) {   // the first step's spread
-        cudaGridDependencySynchronize();
         spread_node(p.csr, r.F1, r, r.fb1, ((int)blockIdx.x - mblocks) * kIbPairThreads + (int)threadIdx.x);
         return;
     }
@@ -750,7 +800,6 @@ ib_pair_batch_kernel(const T* __restrict__ g, const LatticeParams* __restrict__ 
     __shared__ float patch[W][9][(S + 2) * (S + 2)];
     cudaTriggerProgrammaticLaunchCompletion();   // as in ib_pair_kernel
     if ((int)blockIdx.x >= mblocks) {
-        cudaGridDependencySynchronize();
         spread_node(csr, r.F1, r, r.fb1, ((int)blockIdx.x - mblocks) * kIbPairThreads + (int)threadIdx.x);
         return;
     }
@@ -807,12 +856,14 @@ cudaError_t ib_pair_t(int width, const void* g, const LatticeParams& p, const Ib
 }  // namespace
 
 // Nodes per lane.  FP32 below 2^22 nodes: 2, with 40 warps an SM in tiles of 60 x 6
-// (11.5 us a step at 1600 x 800 against 12.1 with 4); above, where fewer
+// (11.6 us a step at 1600 x 800 against 12.2 with 4); above, where fewer
 // instructions per node count for more, 4, with 27 warps in tiles of 120 x 7
-// (233 us at 8192 x 4096 against 241).  16-bit storage: 4 (1600 x 800 11.1 against
-// 11.2, 8192 x 4096 211 against 234).  The outlet column takes its second step
-// from the column before it, which a halo of two nodes does not cover: 4 where
-// nx - 1 starts a tile.
+// (232 us at 8192 x 4096 against 243).  16-bit storage: 4 (1600 x 800 11.1 against
+// 11.4, 8192 x 4096 209 against 239).  Also measured with 4: tiles of 120 x 6 with
+// four blocks an SM (FP32 234, FP16 207 at 8192 x 4096, 11.3 at 1600 x 800), 120 x 8
+// with three (240, 209, 11.4).  The outlet column takes its second step from the
+// column before it, which a halo of two nodes does not cover: 4 where nx - 1
+// starts a tile.
 int pair_npl(int storage, int bcx, int nx, int ny) {
     if (storage != kStoreF32 || (long long)nx * ny >= (1ll << 22)) return 4;
     return bcx == kBcxInout && (nx - 1) % pair_own(2) == 0 ? 4 : 2;

@@ -2,9 +2,8 @@
 same arithmetic node by node, so populations, marker results and body forces are
 equal bit for bit.  Sizes sit at the edges of the kernel's tiles (30 lanes of 2
 or 4 nodes, 6 or 7 rows) and of the vectors; bodies reach the walls, wrap around
-periodic edges and straddle tiles.  The automatic variant takes single steps on
-small FP32 lattices with bodies; there the populations come from a lattice above
-the limit."""
+periodic edges and straddle tiles.  FP32 takes 2 nodes per lane below 2^22 nodes:
+its 4-node form is covered where nx - 1 starts a 60-node tile."""
 import numpy as np
 import pytest
 
@@ -60,7 +59,7 @@ def compare(c, storage, layout=None, steps=(1, 2, 5, 66)):
                                      (W.BCX_CONVECTIVE, W.BCY_NOSLIP), (W.BCX_PERIODIC, W.BCY_NOSLIP)])
 @pytest.mark.parametrize("nx", [118, 119, 120, 121, 122, 124, 128, 129, 240, 241, 363])
 def test_strip_edges(nx, bcx, bcy, storage):
-    ny = 37 if storage != B.BTDF_F32 else 2 ** 17 // nx + 1
+    ny = 37
     bodies = [(nx - 22.3, 18.4, 9.0), (15.2, 20.1, 7.0)]
     if bcx == W.BCX_PERIODIC:
         bodies.append((0.3, 12.0, 6.0))            # wraps in x
@@ -79,7 +78,7 @@ def test_row_edges(ny, bcy):
 def test_deltas_walls_and_layouts(delta, layout):
     # bodies resting on the wall rows, on a strip border (x = 120) and across the periodic y edge
     r = {2: 5.0, 3: 5.5, 4: 6.0, 5: 6.0}[delta]
-    ny = 2 ** 17 // 250 + 1
+    ny = 70
     wall = [(60.3, r + 0.6, 10.0), (120.2, 40.0, 12.0), (200.7, ny - 1 - r, 10.0)]
     for bcy in (W.BCY_FREESLIP, W.BCY_NOSLIP):
         compare(case(250, ny, W.BCX_INOUT, bcy, delta, wall, tau=1.5), B.BTDF_F32, layout)
