@@ -834,35 +834,44 @@ __device__ __forceinline__ void ib_force_body(const T* __restrict__ g, const Lat
     // The populations (previous LBM kernel) and the forces of earlier passes
     // (previous IB kernel) come from the preceding launch: wait for it (a
     // no-op unless this grid was launched as its programmatic dependent),
-    // then let the dependent LBM kernel launch.
+    // then let the dependent LBM kernel launch.  A later pass starts after the
+    // first pass's wait, so the populations are there already and its dependent
+    // may start at once: only the forces of the pass before follow its wait.
+    const bool later = q.F_prev != nullptr;
+    float d[9];
+    SpreadTerms terms;
+    auto gather = [&]() {
+        gather_node<T>(g, p, pull != 0, x, y, d);
+    };
+    if (later) {
+        cudaTriggerProgrammaticLaunchCompletion();
+        terms.load(p.csr, 0, 0);
+        if (act && w != 0.f) {
+            gather();
+            const int seg = __ldg(p.seg_index + (long long)y * p.nseg + x / kSeg);
+            if (seg >= 0) {
+                const int* ptr = p.seg_ptr + (long long)seg * (kSeg + 1) + (x % kSeg);
+                terms.load(p.csr, __ldg(ptr), __ldg(ptr + 1));
+            }
+        }
+    }
     cudaGridDependencySynchronize();
-    cudaTriggerProgrammaticLaunchCompletion();
+    if (!later) cudaTriggerProgrammaticLaunchCompletion();
     float2 Fp = make_float2(0.f, 0.f);
-    if (head && q.F_prev != nullptr) Fp = q.F_prev[m];
+    if (head && later) Fp = q.F_prev[m];
     // Weighted sums over the support (Eq. 14) of the density deviation and
     // of the velocity deviation u* - U_r.
     float wr = 0.f, wu = 0.f, wv = 0.f;
     if (act) {
         if (w != 0.f) {
-            float d[9];
-            gather_node<T>(g, p, pull != 0, x, y, d);
+            if (!later) gather();
             const Moments mo = moments(d, p.urx, p.ury);
             float du = mo.dux, dv = mo.duy;
-            if (q.F_prev != nullptr) {
+            if (later) {
                 // Force field of the earlier passes at this node (Eq. 15) and
                 // the corresponding velocity update (Eq. 11, Algorithm 1 3(d)).
-                const int seg = __ldg(p.seg_index + (long long)y * p.nseg + x / kSeg);
-                float fx = 0.f, fy = 0.f;
-                if (seg >= 0) {
-                    const int* ptr = p.seg_ptr + (long long)seg * (kSeg + 1) + (x % kSeg);
-                    const int b = __ldg(ptr), e = __ldg(ptr + 1);
-                    for (int k = b; k < e; k++) {
-                        const CsrEntry c = p.csr[k];
-                        const float2 F = q.F_prev[c.marker];
-                        fx = __fmaf_rn(c.w, F.x, fx);
-                        fy = __fmaf_rn(c.w, F.y, fy);
-                    }
-                }
+                float fx, fy;
+                terms.sum(p.csr, q.F_prev, fx, fy);
                 du += 0.5f * fx * mo.inv;
                 dv += 0.5f * fy * mo.inv;
             }

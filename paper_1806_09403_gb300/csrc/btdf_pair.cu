@@ -283,43 +283,6 @@ template <int NPL> struct Vec<float, NPL> {
     }
 };
 
-// Spread force (Eq. 15) of the terms b .. e-1.  The first kTerms of them are
-// loaded ahead (no kernel of a step writes them), so that only the loads of the
-// forces, all at once, follow the wait for the kernel that writes those.
-constexpr int kTerms = 8;
-struct SpreadTerms {
-    CsrEntry c[kTerms];
-    int b, e;
-    __device__ __forceinline__ void load(const CsrEntry* csr, int b_, int e_) {
-        b = b_;
-        e = e_;
-#pragma unroll
-        for (int k = 0; k < kTerms; k++) {
-            c[k] = CsrEntry{0, 0.f};
-            if (b + k < e) c[k] = csr[b + k];
-        }
-    }
-    __device__ __forceinline__ void sum(const CsrEntry* csr, const float2* F, float& sx, float& sy) const {
-        float2 f[kTerms];
-#pragma unroll
-        for (int k = 0; k < kTerms; k++) f[k] = b + k < e ? F[c[k].marker] : make_float2(0.f, 0.f);
-        sx = 0.f;
-        sy = 0.f;
-#pragma unroll
-        for (int k = 0; k < kTerms; k++)
-            if (b + k < e) {
-                sx = __fmaf_rn(c[k].w, f[k].x, sx);
-                sy = __fmaf_rn(c[k].w, f[k].y, sy);
-            }
-        for (int k = b + kTerms; k < e; k++) {
-            const CsrEntry t = csr[k];
-            const float2 v = F[t.marker];
-            sx = __fmaf_rn(t.w, v.x, sx);
-            sy = __fmaf_rn(t.w, v.y, sy);
-        }
-    }
-};
-
 // A tile of 30 * NPL columns x TH rows per block.  First step: the block's warps
 // pull the TH + 2 rows of 32 * NPL columns around the tile from memory, collide
 // them and leave the results, rounded to the storage type, in shared memory.
