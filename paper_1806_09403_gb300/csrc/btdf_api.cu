@@ -10,6 +10,7 @@
 #include <cudaTypedefs.h>
 
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -177,6 +178,7 @@ struct btdf_ctx {
     // with spread terms, and the spread forces of either step.
     // Built for the first pair after the markers change, in one allocation.
     void* d_pair = nullptr;
+    bool pair_nomem = false;   // the tables for these markers did not fit: not tried again
     size_t pair_bytes = 0;
     int* d_strip_row = nullptr;
     int4* d_bnodes = nullptr;
@@ -292,6 +294,7 @@ void free_markers(btdf_ctx* ctx) {
     ctx->dev_bytes -= ctx->pair_bytes;
     ctx->pair_bytes = 0;
     dfree(ctx, ctx->d_pair);
+    ctx->pair_nomem = false;
     ctx->d_mk = nullptr;
     ctx->d_aux = nullptr;
     ctx->d_F[0] = ctx->d_F[1] = nullptr;
@@ -519,13 +522,17 @@ bool pairs_allowed(const btdf_ctx* ctx) {
 }
 
 // Tables of the pair kernels for the current markers.
-int ensure_pair_tables(btdf_ctx* ctx) {
+int ensure_pair_tables(btdf_ctx* ctx) try {
     if (ctx->nmark == 0 || ctx->d_pair) return BTDF_OK;
+    if (ctx->pair_nomem) return BTDF_ENOMEM;
     const int nx = ctx->cfg.nx, ny = ctx->cfg.ny;
     const bool px = ctx->cfg.bc_x == kBcxPeriodic;
     const std::vector<int>& seg_ptr = ctx->seg_ptr_host;
     const LatticeParams lp = lattice_params(ctx, ctx->cur);
     const int npl = pair_npl(ctx->cfg.storage, lp.bcx, nx, ny);
+    // slots of the spread arrays are ints; a band segment meets at most 4 strips
+    // (a wrapped narrow lattice's rows are few)
+    if (4ll * (ctx->nband + ny) * 64 * npl > INT_MAX) return fail(ctx, BTDF_ENOMEM, "pair tables too large");
     std::vector<int> strip_row;
     std::vector<int4> bnodes;
     int nsrow = 0;
@@ -557,6 +564,8 @@ int ensure_pair_tables(btdf_ctx* ctx) {
     for (float* fb : ctx->d_fb) CK(cudaMemsetAsync(fb, 0, fb_bytes, st));
     CK(cudaStreamSynchronize(st));
     return BTDF_OK;
+} catch (const std::bad_alloc&) {
+    return fail(ctx, BTDF_ENOMEM, "pair tables do not fit");
 }
 
 // Issues the kernels of two pulling time steps reading buffer `cur`; the state
@@ -1292,6 +1301,13 @@ int btdf_step(btdf_ctx* ctx, int64_t nsteps) {
     int64_t i = 0;
     bool pairs = nsteps - (ctx->poststream ? 1 : 0) >= 2 && pairs_allowed(ctx);
     if (pairs && ctx->nmark > 0 && !ctx->d_pair) {
+        // Building the tables takes the host 0.1-0.3 ms with one body (2-3 ms with
+        // hundreds), a pair saves 2-6 us a step on small lattices and 100 on large
+        // ones: bodies that move every few steps keep single steps.
+        const int64_t worth = (long long)ctx->cfg.nx * ctx->cfg.ny >= (1ll << 22) ? 16 : 64;
+        if (ctx->steps - ctx->hist_from + nsteps < worth) pairs = false;
+    }
+    if (pairs && ctx->nmark > 0 && !ctx->d_pair) {
         // the tables cannot be built while the caller captures the stream
         cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
         if (cudaStreamIsCapturing(ctx->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
@@ -1317,7 +1333,7 @@ int btdf_step(btdf_ctx* ctx, int64_t nsteps) {
                 ctx->cur = 1 - ctx->cur;
             }
         const int rc = ensure_pair_tables(ctx);
-        if (rc == BTDF_ENOMEM) pairs = false;   // single steps need no tables
+        if (rc == BTDF_ENOMEM) pairs = false, ctx->pair_nomem = true;   // single steps need no tables
         else if (rc != BTDF_OK) return rc;
     }
     if (!ctx->prof) {
@@ -1743,9 +1759,9 @@ int btdf_autotune(btdf_ctx* ctx, int32_t steps, int32_t flush_l2, int32_t* chose
                 best = v;
             }
         }
-        if (pairs_possible(ctx) && ctx->grid_override == 0) {   // pairs of steps, as time per step
-            const int rcp = ensure_pair_tables(ctx);
-            if (rcp != BTDF_OK) return rcp;
+        const int rcp = pairs_possible(ctx) && ctx->grid_override == 0 ? ensure_pair_tables(ctx) : BTDF_ENOMEM;
+        if (rcp != BTDF_OK && rcp != BTDF_ENOMEM) return rcp;
+        if (rcp == BTDF_OK) {   // pairs of steps, as time per step
             for (int i = 0; i < steps + 2; i++) {
                 if (flush) CK(launch_l2_flush(flush, l2_flush_bytes(), st));
                 const int e = std::max(i - 2, 0);

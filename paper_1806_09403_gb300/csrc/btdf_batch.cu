@@ -6,6 +6,7 @@
 #include "btdf_internal.cuh"
 
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <cstring>
 #include <new>
@@ -79,6 +80,7 @@ struct btdf_batch {
     std::vector<std::vector<int>> band_keys, seg_ptr;   // per lattice, for those tables
     std::vector<size_t> cs_off;
     void* d_pair = nullptr;
+    bool pair_nomem = false;   // the tables for these markers did not fit: not tried again
     float2* d_F1 = nullptr;
     PairForces pf{};
     PairBatch pb{};
@@ -125,6 +127,7 @@ void free_marker_data(btdf_batch* bt) {
     bfree(bt->d_seg_ptr);
     bfree(bt->d_csr);
     bfree(bt->d_pair);
+    bt->pair_nomem = false;
     bfree(bt->d_body_ptr);
     bfree(bt->d_body_scale);
     bfree(bt->d_hist);
@@ -343,13 +346,18 @@ int rebuild(btdf_batch* bt) {
 }
 
 // Tables of the pair kernels, for the first pair after the markers were set.
-int ensure_pair_tables(btdf_batch* bt) {
+int ensure_pair_tables(btdf_batch* bt) try {
     if (bt->d_pair) return BTDF_OK;
+    if (bt->pair_nomem) return BTDF_ENOMEM;
     long long nodes_all = 0;
     int npl = 2;
     for (int c = 0; c < bt->n; c++) nodes_all += (long long)bt->cfg[c].nx * bt->cfg[c].ny;
     for (int c = 0; c < bt->n; c++)
         if (nodes_all >= (1ll << 22) || pair_npl(bt->storage, bt->cfg[c].bc_x, bt->cfg[c].nx, bt->cfg[c].ny) == 4) npl = 4;
+    long long bands = 0;   // slots of the spread arrays are ints, as for one lattice
+    for (int c = 0; c < bt->n && bt->nmark > 0; c++)
+        bands += (long long)bt->band_keys[c].size() + bt->cfg[c].ny;
+    if (4ll * bands * 64 * npl > INT_MAX) return bfail(bt, BTDF_ENOMEM, "pair tables too large");
     std::vector<int> strip_row;
     std::vector<int4> nodes, tiles;
     std::vector<PairLattice> lat(bt->n);
@@ -416,6 +424,8 @@ int ensure_pair_tables(btdf_batch* bt) {
     b.ntile = (int)tiles.size();
     bt->pb = b;
     return BTDF_OK;
+} catch (const std::bad_alloc&) {
+    return bfail(bt, BTDF_ENOMEM, "pair tables do not fit");
 }
 
 // Pairs of steps unless a launch shape was chosen: with every support inside.
@@ -784,9 +794,9 @@ int btdf_batch_autotune(btdf_batch* bt, int32_t steps, int32_t flush_l2, int32_t
             res[v] = interquartile_mean(t);
             if (v == 1 || res[v] < res[best]) best = v;
         }
-        if (bt->nmark == 0 || bt->markers_inside) {   // pairs of steps, as time per step
-            const int rcp = ensure_pair_tables(bt);
-            if (rcp != BTDF_OK) return rcp;
+        const int rcp = bt->nmark == 0 || bt->markers_inside ? ensure_pair_tables(bt) : BTDF_ENOMEM;
+        if (rcp != BTDF_OK && rcp != BTDF_ENOMEM) return rcp;
+        if (rcp == BTDF_OK) {   // pairs of steps, as time per step
             for (int i = 0; i < steps + 2; i++) {
                 if (flush) BCK(launch_l2_flush(flush, l2_flush_bytes(), st));
                 const int e = std::max(i - 2, 0);
@@ -847,7 +857,7 @@ int btdf_batch_step(btdf_batch* bt, int64_t nsteps) {
             pairs = false;
         } else {
             const int rc = ensure_pair_tables(bt);
-            if (rc == BTDF_ENOMEM) pairs = false;
+            if (rc == BTDF_ENOMEM) pairs = false, bt->pair_nomem = true;
             else if (rc != BTDF_OK) return rc;
         }
     }

@@ -34,11 +34,6 @@
 namespace btdf {
 namespace {
 
-template <typename T> struct Raw16;
-template <> struct Raw16<__half> : Raw<__half> {};
-template <> struct Raw16<__nv_bfloat16> : Io16<__nv_bfloat16, __nv_bfloat162> {};
-
-
 // Two FP32 values in a 64-bit register, and the packed operations on them (two
 // IEEE round-to-nearest operations each).  Held as 64-bit values throughout:
 // with float2 the compiler re-pairs operands with moves.
@@ -553,8 +548,9 @@ pair_kernel(const T* __restrict__ gin, T* __restrict__ gout, const __grid_consta
         if (p.nbody > 0) cudaGridDependencySynchronize();
         const unsigned long long step = p.step != nullptr ? *p.step : 0ull;
         const int half = NW / 2, w = (int)threadIdx.x >> 5;
-        if (w < half) body_forces(p, q.F1, step, blockIdx.x * half + w, nred * half);
-        else if (w < 2 * half) body_forces(p, p.F, step + 1ull, blockIdx.x * half + w - half, nred * half);
+        // a ring of one step keeps the second step's forces only
+        if (w < half && p.hist_len > 1) body_forces(p, q.F1, step, blockIdx.x * half + w, nred * half);
+        if (w >= half && w < 2 * half) body_forces(p, p.F, step + 1ull, blockIdx.x * half + w - half, nred * half);
         pair_finish(p.step, step, q.done, nred);
         return;
     }
@@ -576,10 +572,10 @@ pair_batch_kernel(const T* __restrict__ gin, T* __restrict__ gout, const __grid_
         if (b.nbody > 0) cudaGridDependencySynchronize();
         const unsigned long long step = *b.step;
         const int half = NW / 2, w = (int)threadIdx.x >> 5;
-        if (w < half)
+        if (w < half && b.hist_len > 1)   // as in pair_kernel
             body_forces(b.nbody, b.body_rng, 2, b.body_scale, b.hist, b.hist_len, q.F1, step, blockIdx.x * half + w,
                         nred * half);
-        else if (w < 2 * half)
+        if (w >= half && w < 2 * half)
             body_forces(b.nbody, b.body_rng, 2, b.body_scale, b.hist, b.hist_len, b.F2, step + 1ull,
                         blockIdx.x * half + w - half, nred * half);
         pair_finish(b.step, step, q.done, nred);

@@ -35,7 +35,9 @@ def case(nx, ny, bcx, bcy, delta=3, bodies=(), gx=0.0, tau=0.6):
     return c
 
 
-def compare(c, storage, layout=None, steps=(1, 2, 5, 66)):
+# Pairs start once enough steps of the same markers make up for their tables
+# (64, or one call of as many); every run below ends with pairs in short calls.
+def compare(c, storage, layout=None, steps=(1, 2, 66, 2, 5)):
     a = B.Lattice.from_case(c, storage=storage, layout=layout, history_len=16)
     b = B.Lattice.from_case(c, storage=storage, layout=layout, history_len=16)
     b.tune(1)
@@ -94,7 +96,7 @@ def test_clipped_supports_take_single_steps():
 def test_larger_lattice_and_many_bodies():
     bodies = [(40.0 + 37.0 * i + 0.31 * j, 30.0 + 33.0 * j + 0.17 * i, 14.0) for i in range(12) for j in range(8)]
     for storage in STORAGES:
-        compare(case(499, 301, W.BCX_INOUT, W.BCY_FREESLIP, 3, bodies), storage, steps=(2, 131))
+        compare(case(499, 301, W.BCX_INOUT, W.BCY_FREESLIP, 3, bodies), storage, steps=(2, 131, 4))
 
 
 @pytest.mark.parametrize("storage", STORAGES)
@@ -127,3 +129,19 @@ def test_batch_pairs(storage):
         for k in range(len(a.bodies)):
             fa, fb = (x.forces(k, x.steps - min(n, 8), min(n, 8)) for x in (a, b))
             assert np.array_equal(fa[0], fb[0]) and np.array_equal(fa[1], fb[1]), (n, k)
+
+
+def test_history_of_one_step_and_moved_markers():
+    # a ring of one step keeps the last step's forces; moved markers rebuild the tables
+    c = case(150, 61, W.BCX_INOUT, W.BCY_FREESLIP, bodies=[(60.3, 30.2, 9.0)])
+    a = B.Lattice.from_case(c, history_len=1)
+    b = B.Lattice.from_case(c, history_len=1)
+    b.tune(1)
+    for move, n in ((0.0, 80), (0.4, 2), (0.4, 70), (0.9, 3), (0.9, 64), (0.9, 4)):
+        for x in (a, b):
+            if move:
+                x.move_markers(0, c.bodies[0].X + move, c.bodies[0].Y)
+            x.step(n)
+        fa, fb = a.forces(0, a.steps - 1, 1), b.forces(0, b.steps - 1, 1)
+        assert np.array_equal(fa[0], fb[0]) and np.array_equal(fa[1], fb[1])
+        assert np.array_equal(a.field(B.FIELD_POPS), b.field(B.FIELD_POPS))
