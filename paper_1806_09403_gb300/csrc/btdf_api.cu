@@ -178,6 +178,7 @@ struct btdf_ctx {
     // with spread terms, and the spread forces of either step.
     // Built for the first pair after the markers change, in one allocation.
     void* d_pair = nullptr;
+    int64_t marker_steps = 0;   // steps taken with these markers
     bool pair_nomem = false;   // the tables for these markers did not fit: not tried again
     size_t pair_bytes = 0;
     int* d_strip_row = nullptr;
@@ -295,6 +296,7 @@ void free_markers(btdf_ctx* ctx) {
     ctx->pair_bytes = 0;
     dfree(ctx, ctx->d_pair);
     ctx->pair_nomem = false;
+    ctx->marker_steps = 0;
     ctx->d_mk = nullptr;
     ctx->d_aux = nullptr;
     ctx->d_F[0] = ctx->d_F[1] = nullptr;
@@ -1302,10 +1304,13 @@ int btdf_step(btdf_ctx* ctx, int64_t nsteps) {
     bool pairs = nsteps - (ctx->poststream ? 1 : 0) >= 2 && pairs_allowed(ctx);
     if (pairs && ctx->nmark > 0 && !ctx->d_pair) {
         // Building the tables takes the host 0.1-0.3 ms with one body (2-3 ms with
-        // hundreds), a pair saves 2-6 us a step on small lattices and 100 on large
-        // ones: bodies that move every few steps keep single steps.
-        const int64_t worth = (long long)ctx->cfg.nx * ctx->cfg.ny >= (1ll << 22) ? 16 : 64;
-        if (ctx->steps - ctx->hist_from + nsteps < worth) pairs = false;
+        // hundreds); a pair saves 2-6 us a step on small lattices, and on large ones
+        // 100 in FP32 but 11 in 16-bit storage.  So bodies that move every few steps
+        // keep single steps, and the tables are built once the markers have been used
+        // for about as many steps as pay for them.
+        const bool large = (long long)ctx->cfg.nx * ctx->cfg.ny >= (1ll << 22);
+        const int64_t worth = !large ? 64 : ctx->cfg.storage == kStoreF32 ? 16 : 256;
+        if (ctx->marker_steps + nsteps < worth) pairs = false;
     }
     if (pairs && ctx->nmark > 0 && !ctx->d_pair) {
         // the tables cannot be built while the caller captures the stream
@@ -1353,6 +1358,7 @@ int btdf_step(btdf_ctx* ctx, int64_t nsteps) {
         i += two ? 2 : 1;
     }
     ctx->steps += nsteps;
+    ctx->marker_steps += nsteps;
     return BTDF_OK;
 }
 
