@@ -194,7 +194,11 @@ int btdf_set_inflow(btdf_ctx *ctx, double u_in);
 int btdf_move_markers(btdf_ctx *ctx, int32_t body, const double *X, const double *Y);
 
 /* Advances nsteps time steps (Algorithm 1), asynchronously on the context
- * stream.  Requires btdf_init_fields or btdf_load_state first (ESTATE). */
+ * stream.  Requires btdf_init_fields or btdf_load_state first (ESTATE).
+ * A call that the caller captures into a CUDA graph keeps its parity: an even
+ * number of steps ends in the population buffer it began with, so that replays
+ * advance (after the first step since btdf_init_fields or a post-streaming
+ * checkpoint; the host's step counter does not follow replays). */
 int btdf_step(btdf_ctx *ctx, int64_t nsteps);
 
 /* Waits for the context stream and returns the sticky device status

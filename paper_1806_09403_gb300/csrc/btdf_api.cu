@@ -82,7 +82,7 @@ using namespace btdf;
 
 namespace {
 
-constexpr int kGraphSteps = 64;          // steps per replayed CUDA graph (even)
+constexpr int kGraphSteps = 64;          // steps per replayed CUDA graph (a multiple of 4: an even number of pairs)
 constexpr int kFullGrid = 1 << 30;       // grid cap meaning "one row segment per warp"
 constexpr int kSchedWords = 3;           // device counters: the two of LatticeParams.sched, pair_kernel's
 constexpr int kStageSlots = 4;           // pinned staging slots for marker velocities
@@ -1312,14 +1312,9 @@ int btdf_step(btdf_ctx* ctx, int64_t nsteps) {
         const int64_t worth = !large ? 64 : ctx->cfg.storage == kStoreF32 ? 16 : 256;
         if (ctx->marker_steps + nsteps < worth) pairs = false;
     }
-    if (pairs && ctx->nmark > 0 && !ctx->d_pair) {
-        // the tables cannot be built while the caller captures the stream
-        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-        if (cudaStreamIsCapturing(ctx->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
-            cudaGetLastError();
-            pairs = false;
-        }
-    }
+    const bool captured = pairs && stream_captures(ctx->stream);
+    // the tables cannot be built while the caller captures the stream
+    if (captured && ctx->nmark > 0 && !ctx->d_pair) pairs = false;
     if (nsteps > 0 && ctx->poststream) {
         const int rc = enqueue_step(ctx, ctx->stream, false, ctx->cur, ctx->prof);
         if (rc != BTDF_OK) return rc;
@@ -1349,8 +1344,9 @@ int btdf_step(btdf_ctx* ctx, int64_t nsteps) {
             i += kGraphSteps;
         }
     }
+    int64_t npairs = pairs ? pairs_of(nsteps - i, captured) : 0;
     while (i < nsteps) {
-        const bool two = pairs && nsteps - i >= 2;
+        const bool two = npairs-- > 0;
         const int rc = two ? enqueue_pair(ctx, ctx->stream, ctx->cur)
                            : enqueue_step(ctx, ctx->stream, true, ctx->cur, ctx->prof);
         if (rc != BTDF_OK) return rc;

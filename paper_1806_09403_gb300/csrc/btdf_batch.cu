@@ -17,7 +17,7 @@ using namespace btdf;
 
 namespace {
 
-constexpr int kBatchGraphSteps = 32;
+constexpr int kBatchGraphSteps = 32;   // a multiple of 4: an even number of pairs
 
 struct BBody {
     int first = 0, n = 0, lattice = 0;
@@ -849,11 +849,10 @@ int btdf_batch_step(btdf_batch* bt, int64_t nsteps) {
         if (!bt->has_fields[c]) return bfail(bt, BTDF_ESTATE, "every lattice needs btdf_batch_init_fields");
     int64_t i = 0;
     bool pairs = nsteps - (bt->poststream ? 1 : 0) >= 2 && pairs_allowed(bt);
+    const bool captured = pairs && stream_captures(bt->stream);
     if (pairs && !bt->d_pair) {
         // no tables while the caller captures the stream; single steps need none
-        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-        if (cudaStreamIsCapturing(bt->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
-            cudaGetLastError();
+        if (captured) {
             pairs = false;
         } else {
             const int rc = ensure_pair_tables(bt);
@@ -874,8 +873,9 @@ int btdf_batch_step(btdf_batch* bt, int64_t nsteps) {
         BCK(cudaGraphLaunch(bt->gexec[bt->cur], bt->stream));
         i += kBatchGraphSteps;
     }
+    int64_t npairs = pairs ? pairs_of(nsteps - i, captured) : 0;
     while (i < nsteps) {
-        const bool two = pairs && nsteps - i >= 2;
+        const bool two = npairs-- > 0;
         const int rc = two ? enqueue_pair(bt, bt->stream, bt->cur) : enqueue(bt, bt->stream, true, bt->cur);
         if (rc != BTDF_OK) return rc;
         bt->cur = 1 - bt->cur;

@@ -278,6 +278,19 @@ void build_pair_tables(int nx, int ny, int nseg, bool px, int npl, int nstrip, c
                        const std::vector<int>& seg_ptr, int term0, std::vector<int>& strip_row,
                        std::vector<int4>& nodes, int& nsrow);
 
+// Whether the caller captures the stream (or that cannot be told).
+inline bool stream_captures(cudaStream_t st) {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cs) == cudaSuccess) return cs != cudaStreamCaptureStatusNone;
+    cudaGetLastError();
+    return true;
+}
+// How many of n steps go in pairs.  A pair changes the population buffer once
+// for two steps; in a call that the caller captures the pairs are even in
+// number, so that an even count of steps ends in the buffer it began with, as
+// single steps do, and a replay of the capture goes on from the one before.
+inline int64_t pairs_of(int64_t n, bool captured) { return captured ? n / 4 * 2 : n / 2; }
+
 // Two pulling steps in one kernel.
 cudaError_t launch_pair(int storage, const void* gin, void* gout, const LatticeParams& p, const PairForces& q,
                         bool pdl, cudaStream_t st);
