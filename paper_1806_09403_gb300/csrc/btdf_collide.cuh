@@ -81,12 +81,13 @@ __device__ __forceinline__ void body_forces(const LatticeParams& p, const float2
 // f holds the post-streaming deviations of NPL nodes at their stored scale,
 // (Fx, Fy) the force density of the spread (Eq. 15), without the uniform body
 // force; forced: any of them, or the uniform force, is not zero.  Calls
-// store(a, o) with the NPL post-collision values of population a (stored
-// scale), one population after the other.
-template <typename T, int NPL, typename Store>
+// begin() between the moments and the collision, then store(a, o) with the NPL
+// post-collision values of population a (stored scale), one population after
+// the other.
+template <typename T, int NPL, typename Begin, typename Store>
 __device__ __forceinline__ void collide_nodes(const float (&f)[9][NPL], const LatticeParams& p,
                                               float (&Fx)[NPL], float (&Fy)[NPL], bool forced,
-                                              Store&& store) {
+                                              Begin&& begin, Store&& store) {
     // Moments (Eqs. 9-10) and the velocity correction u = u* + f / (2 rho)
     // (Eq. 11), as deviations from the reference state.
     float drho[NPL], rho[NPL], du[NPL], dv[NPL], pd0[NPL], uF[NPL], inv[NPL];
@@ -140,6 +141,7 @@ __device__ __forceinline__ void collide_nodes(const float (&f)[9][NPL], const La
         }
     };
 
+    begin();
     // Collision (Eqs. 5-7), one population at a time, in the form
     //   d_eq / w = drho (1 + P(U_r)) + rho (P(u) - P(U_r))
     //   P(u) - P(U_r) = ed (3 + 9 e.U_r + 4.5 ed) - 1.5 (2 U_r.du + du^2),  ed = e.du

@@ -109,11 +109,26 @@ __device__ __forceinline__ void collide_store(float (&f)[9][NPL], T* __restrict_
         }
     }
 
-    T* const out = gout + rowoff;
-    const bool store = live && x0 < p.nx;
-    collide_nodes<T, NPL>(f, p, Fx, Fy, forced, [&](int a, const float (&o)[NPL]) {
-        if (store) Raw<T>::template stv<NPL>(out + p.poff[a], o);
-    });
+    // With 2 nodes per lane the output address is formed after the moments: held
+    // across them it changes the order of the loads, and FP32 on 4096 x 2048 takes
+    // 103 us a step instead of 90 (2048 x 2048 54.6 instead of 48.4).  With 4 and 1
+    // formed early: 88.5 and 135 us against 88.9 and 135, FP16 with 4 62.6 against
+    // 63.6.
+    constexpr bool late = NPL == 2;
+    T* out = nullptr;
+    bool store = false;
+    auto place = [&]() {
+        out = gout + rowoff;
+        store = live && x0 < p.nx;
+    };
+    if (!late) place();
+    collide_nodes<T, NPL>(f, p, Fx, Fy, forced,
+                          [&]() {
+                              if (late) place();
+                          },
+                          [&](int a, const float (&o)[NPL]) {
+                              if (store) Raw<T>::template stv<NPL>(out + p.poff[a], o);
+                          });
 }
 
 // One row segment of 32 * NPL nodes: NPL consecutive nodes per lane.  All

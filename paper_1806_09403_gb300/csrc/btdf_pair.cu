@@ -685,7 +685,7 @@ __device__ __forceinline__ void ib_pair_marker(const T* __restrict__ g, const La
         float Fx[1], Fy[1];
         terms[k].sum(p.csr, F1, Fx[0], Fy[0]);
         const bool forced = band[k] || p.gx != 0.f || p.gy != 0.f;
-        collide_nodes<T, 1>(f[k], p, Fx, Fy, forced, [&](int a, const float (&o)[1]) {
+        collide_nodes<T, 1>(f[k], p, Fx, Fy, forced, []() {}, [&](int a, const float (&o)[1]) {
             T st;
             Raw<T>::template stv<1>(&st, o);
             patch[a][e] = Io<T>::ld1s(&st);
