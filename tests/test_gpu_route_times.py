@@ -52,3 +52,15 @@ def test_two_node_register_kernel_streams_like_the_four_node_one():
         x.tune(v)
     two, four = lowest([lambda x=x: x.step(64) for x in lats])
     assert two < 1.06 * four, (two, four)
+
+
+@pytest.mark.parametrize("nx,ny,storage,bcx,single", [
+    # the outlet column's nine loads on one path (12% slower than single steps one by one)
+    (160, 80, B.BTDF_F32, W.BCX_CONVECTIVE, 2),
+    (320, 160, B.BTDF_F32, W.BCX_CONVECTIVE, 2),
+])
+def test_automatic_steps_are_not_slower_than_single_ones(nx, ny, storage, bcx, single):
+    lats = [lattice(nx, ny, storage, bcx) for _ in range(2)]
+    lats[1].tune(single)
+    auto, one = lowest([lambda x=x: x.step(512) for x in lats])
+    assert auto < 1.04 * one, (auto, one)
