@@ -194,7 +194,12 @@ int btdf_set_inflow(btdf_ctx *ctx, double u_in);
 int btdf_move_markers(btdf_ctx *ctx, int32_t body, const double *X, const double *Y);
 
 /* Advances nsteps time steps (Algorithm 1), asynchronously on the context
- * stream.  Requires btdf_init_fields or btdf_load_state first (ESTATE).
+ * stream: the call never waits for the stream.  Requires btdf_init_fields or
+ * btdf_load_state first (ESTATE).  The call in which steps first go in pairs
+ * (btdf_tune, variant 0) after markers were added or moved builds their tables on
+ * the host (0.1 ms with one body, a few ms with hundreds) and allocates device and
+ * page-locked memory for them; where that cannot be had the steps are taken
+ * singly.  After an error the step counter holds the steps that were issued.
  * A call that the caller captures into a CUDA graph keeps its parity: an even
  * number of steps ends in the population buffer it began with, so that replays
  * advance (after the first step since btdf_init_fields or a post-streaming
@@ -409,6 +414,7 @@ int btdf_batch_tune(btdf_batch *b, int32_t variant);
 /* As btdf_autotune, over the batch's launch shapes 1..4; ms[0..4], ms[0] being
  * half the time of a pair of steps (-1 where pairs cannot run). */
 int btdf_batch_autotune(btdf_batch *b, int32_t steps, int32_t flush_l2, int32_t *chosen, float *ms);
+/* As btdf_step, for every lattice. */
 int btdf_batch_step(btdf_batch *b, int64_t nsteps);
 int btdf_batch_sync(btdf_batch *b);
 int64_t btdf_batch_step_count(const btdf_batch *b);

@@ -177,7 +177,7 @@ struct btdf_ctx {
     // Pairs of steps (PairForces): the band rows of the strip pairs, their nodes
     // with spread terms, and the spread forces of either step.
     // Built for the first pair after the markers change, in one allocation.
-    void* d_pair = nullptr;
+    PairMemory pair;
     int64_t marker_steps = 0;   // steps taken with these markers
     bool pair_nomem = false;   // the tables for these markers did not fit: not tried again
     size_t pair_bytes = 0;
@@ -294,7 +294,7 @@ void free_markers(btdf_ctx* ctx) {
     dfree(ctx, ctx->d_arena);
     ctx->dev_bytes -= ctx->pair_bytes;
     ctx->pair_bytes = 0;
-    dfree(ctx, ctx->d_pair);
+    pair_memory_free(ctx->pair);
     ctx->pair_nomem = false;
     ctx->marker_steps = 0;
     ctx->d_mk = nullptr;
@@ -523,9 +523,12 @@ bool pairs_allowed(const btdf_ctx* ctx) {
     return ctx->variant == kVarAuto && ctx->grid_override == 0 ? true : ctx->pairs_tuned;
 }
 
-// Tables of the pair kernels for the current markers.
+// Tables of the pair kernels for the current markers, built by the host and
+// uploaded in stream order: the caller does not wait for the stream.  BTDF_ENOMEM
+// where they cannot be had (then, or ever for these markers: pair_nomem); steps
+// need none singly.
 int ensure_pair_tables(btdf_ctx* ctx) try {
-    if (ctx->nmark == 0 || ctx->d_pair) return BTDF_OK;
+    if (ctx->nmark == 0 || ctx->pair.dev) return BTDF_OK;
     if (ctx->pair_nomem) return BTDF_ENOMEM;
     const int nx = ctx->cfg.nx, ny = ctx->cfg.ny;
     const bool px = ctx->cfg.bc_x == kBcxPeriodic;
@@ -534,7 +537,10 @@ int ensure_pair_tables(btdf_ctx* ctx) try {
     const int npl = pair_npl(ctx->cfg.storage, lp.bcx, nx, ny);
     // slots of the spread arrays are ints; a band segment meets at most 4 strips
     // (a wrapped narrow lattice's rows are few)
-    if (4ll * (ctx->nband + ny) * 64 * npl > INT_MAX) return fail(ctx, BTDF_ENOMEM, "pair tables too large");
+    if (4ll * (ctx->nband + ny) * 64 * npl > INT_MAX) {
+        ctx->pair_nomem = true;
+        return BTDF_ENOMEM;
+    }
     std::vector<int> strip_row;
     std::vector<int4> bnodes;
     int nsrow = 0;
@@ -544,30 +550,32 @@ int ensure_pair_tables(btdf_ctx* ctx) try {
     Arena A;
     const size_t o_srow = A.take<int>(sizeof(int) * strip_row.size());
     const size_t o_bn = A.take<int4>(sizeof(int4) * std::max<size_t>(bnodes.size(), 1));
-    const size_t o_fb0 = A.take<float>(fb_bytes);
+    const size_t o_fb0 = A.take<float>(fb_bytes);   // band nodes without terms keep a zero force
     const size_t o_fb1 = A.take<float>(fb_bytes);
-    const size_t before = ctx->dev_bytes;
-    const cudaError_t ea = dalloc(ctx, &ctx->d_pair, A.size);
-    if (ea != cudaSuccess)
-        return ea == cudaErrorMemoryAllocation ? fail(ctx, BTDF_ENOMEM, "pair tables do not fit")
-                                               : cuda_fail(ctx, ea, "cudaMalloc");
-    ctx->pair_bytes = ctx->dev_bytes - before;
-    char* base = (char*)ctx->d_pair;
+    const cudaError_t ea = pair_memory_alloc(ctx->pair, A.size, o_fb0);
+    if (ea != cudaSuccess) {
+        ctx->pair_nomem = ea == cudaErrorMemoryAllocation;
+        return BTDF_ENOMEM;
+    }
+    memcpy((char*)ctx->pair.pin + o_srow, strip_row.data(), sizeof(int) * strip_row.size());
+    if (!bnodes.empty()) memcpy((char*)ctx->pair.pin + o_bn, bnodes.data(), sizeof(int4) * bnodes.size());
+    const cudaError_t eu = pair_memory_upload(ctx->pair, A.size, o_fb0, ctx->stream);
+    if (eu != cudaSuccess) {
+        pair_memory_free(ctx->pair);
+        return cuda_fail(ctx, eu, "uploading the pair tables");
+    }
+    ctx->dev_bytes += A.size;
+    ctx->pair_bytes = A.size;
+    char* base = (char*)ctx->pair.dev;
     ctx->d_strip_row = (int*)(base + o_srow);
     ctx->d_bnodes = (int4*)(base + o_bn);
     ctx->nbnode = (int)bnodes.size();
     ctx->d_fb[0] = (float*)(base + o_fb0);
     ctx->d_fb[1] = (float*)(base + o_fb1);
-    cudaStream_t st = ctx->stream;
-    CK(cudaMemcpyAsync(ctx->d_strip_row, strip_row.data(), sizeof(int) * strip_row.size(), cudaMemcpyHostToDevice, st));
-    if (!bnodes.empty())
-        CK(cudaMemcpyAsync(ctx->d_bnodes, bnodes.data(), sizeof(int4) * bnodes.size(), cudaMemcpyHostToDevice, st));
-    // band nodes without terms keep a zero force
-    for (float* fb : ctx->d_fb) CK(cudaMemsetAsync(fb, 0, fb_bytes, st));
-    CK(cudaStreamSynchronize(st));
     return BTDF_OK;
 } catch (const std::bad_alloc&) {
-    return fail(ctx, BTDF_ENOMEM, "pair tables do not fit");
+    ctx->pair_nomem = true;
+    return BTDF_ENOMEM;
 }
 
 // Issues the kernels of two pulling time steps reading buffer `cur`; the state
@@ -1300,9 +1308,15 @@ int btdf_step(btdf_ctx* ctx, int64_t nsteps) {
     if (!ctx) return BTDF_EINVAL;
     if (nsteps < 0) return fail(ctx, BTDF_EINVAL, "nsteps < 0");
     if (!ctx->has_fields) return fail(ctx, BTDF_ESTATE, "call btdf_init_fields or btdf_load_state first");
-    int64_t i = 0;
+    int64_t i = 0;   // steps issued so far
+    // what has been issued counts, also where the rest cannot be
+    auto stop = [&](int rc) {
+        ctx->steps += i;
+        ctx->marker_steps += i;
+        return rc;
+    };
     bool pairs = nsteps - (ctx->poststream ? 1 : 0) >= 2 && pairs_allowed(ctx);
-    if (pairs && ctx->nmark > 0 && !ctx->d_pair) {
+    if (pairs && ctx->nmark > 0 && !ctx->pair.dev) {
         // Building the tables takes the host 0.1-0.3 ms with one body (2-3 ms with
         // hundreds); a pair saves 2-6 us a step on small lattices, and on large ones
         // 100 in FP32 but 11 in 16-bit storage.  So bodies that move every few steps
@@ -1314,7 +1328,7 @@ int btdf_step(btdf_ctx* ctx, int64_t nsteps) {
     }
     const bool captured = pairs && stream_captures(ctx->stream);
     // the tables cannot be built while the caller captures the stream
-    if (captured && ctx->nmark > 0 && !ctx->d_pair) pairs = false;
+    if (captured && ctx->nmark > 0 && !ctx->pair.dev) pairs = false;
     if (nsteps > 0 && ctx->poststream) {
         const int rc = enqueue_step(ctx, ctx->stream, false, ctx->cur, ctx->prof);
         if (rc != BTDF_OK) return rc;
@@ -1326,21 +1340,22 @@ int btdf_step(btdf_ctx* ctx, int64_t nsteps) {
         // The tables of the pair kernels take the host 2-3 ms with hundreds of
         // bodies: on a large lattice a few single steps keep the device busy
         // meanwhile.
-        if (ctx->nmark > 0 && !ctx->d_pair && (long long)ctx->cfg.nx * ctx->cfg.ny >= (1ll << 23))
+        if (ctx->nmark > 0 && !ctx->pair.dev && (long long)ctx->cfg.nx * ctx->cfg.ny >= (1ll << 23))
             for (int k = 0; k < 6 && i < nsteps; k++, i++) {
                 const int rc = enqueue_step(ctx, ctx->stream, true, ctx->cur, false);
-                if (rc != BTDF_OK) return rc;
+                if (rc != BTDF_OK) return stop(rc);
                 ctx->cur = 1 - ctx->cur;
             }
         const int rc = ensure_pair_tables(ctx);
-        if (rc == BTDF_ENOMEM) pairs = false, ctx->pair_nomem = true;   // single steps need no tables
-        else if (rc != BTDF_OK) return rc;
+        if (rc == BTDF_ENOMEM) pairs = false;   // single steps need no tables
+        else if (rc != BTDF_OK) return stop(rc);
     }
     if (!ctx->prof) {
         while (nsteps - i >= kGraphSteps) {
             const int rc = ensure_graph(ctx, ctx->cur, pairs);
-            if (rc != BTDF_OK) return rc;
-            CK(cudaGraphLaunch(ctx->gexec[ctx->cur], ctx->stream));
+            if (rc != BTDF_OK) return stop(rc);
+            const cudaError_t e = cudaGraphLaunch(ctx->gexec[ctx->cur], ctx->stream);
+            if (e != cudaSuccess) return stop(cuda_fail(ctx, e, "cudaGraphLaunch"));
             i += kGraphSteps;
         }
     }
@@ -1349,13 +1364,11 @@ int btdf_step(btdf_ctx* ctx, int64_t nsteps) {
         const bool two = npairs-- > 0;
         const int rc = two ? enqueue_pair(ctx, ctx->stream, ctx->cur)
                            : enqueue_step(ctx, ctx->stream, true, ctx->cur, ctx->prof);
-        if (rc != BTDF_OK) return rc;
+        if (rc != BTDF_OK) return stop(rc);
         ctx->cur = 1 - ctx->cur;
         i += two ? 2 : 1;
     }
-    ctx->steps += nsteps;
-    ctx->marker_steps += nsteps;
-    return BTDF_OK;
+    return stop(BTDF_OK);
 }
 
 int btdf_sync(btdf_ctx* ctx) {

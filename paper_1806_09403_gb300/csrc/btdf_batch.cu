@@ -79,7 +79,7 @@ struct btdf_batch {
     bool markers_inside = true;
     std::vector<std::vector<int>> band_keys, seg_ptr;   // per lattice, for those tables
     std::vector<size_t> cs_off;
-    void* d_pair = nullptr;
+    PairMemory pair;
     bool pair_nomem = false;   // the tables for these markers did not fit: not tried again
     float2* d_F1 = nullptr;
     PairForces pf{};
@@ -126,7 +126,7 @@ void free_marker_data(btdf_batch* bt) {
     bfree(bt->d_seg_index);
     bfree(bt->d_seg_ptr);
     bfree(bt->d_csr);
-    bfree(bt->d_pair);
+    pair_memory_free(bt->pair);
     bt->pair_nomem = false;
     bfree(bt->d_body_ptr);
     bfree(bt->d_body_scale);
@@ -345,9 +345,10 @@ int rebuild(btdf_batch* bt) {
     return upload_descs(bt);
 }
 
-// Tables of the pair kernels, for the first pair after the markers were set.
+// Tables of the pair kernels, for the first pair after the markers were set; as for
+// one lattice, the caller does not wait for the stream.
 int ensure_pair_tables(btdf_batch* bt) try {
-    if (bt->d_pair) return BTDF_OK;
+    if (bt->pair.dev) return BTDF_OK;
     if (bt->pair_nomem) return BTDF_ENOMEM;
     long long nodes_all = 0;
     int npl = 2;
@@ -357,7 +358,10 @@ int ensure_pair_tables(btdf_batch* bt) try {
     long long bands = 0;   // slots of the spread arrays are ints, as for one lattice
     for (int c = 0; c < bt->n && bt->nmark > 0; c++)
         bands += (long long)bt->band_keys[c].size() + bt->cfg[c].ny;
-    if (4ll * bands * 64 * npl > INT_MAX) return bfail(bt, BTDF_ENOMEM, "pair tables too large");
+    if (4ll * bands * 64 * npl > INT_MAX) {
+        bt->pair_nomem = true;
+        return BTDF_ENOMEM;
+    }
     std::vector<int> strip_row;
     std::vector<int4> nodes, tiles;
     std::vector<PairLattice> lat(bt->n);
@@ -384,13 +388,13 @@ int ensure_pair_tables(btdf_batch* bt) try {
                  b_row = up(sizeof(int) * std::max<size_t>(strip_row.size(), 1)),
                  b_node = up(sizeof(int4) * std::max<size_t>(nodes.size(), 1)), b_fb = up(fb),
                  b_F = up(sizeof(float2) * std::max(bt->nmark, 1));
-    const cudaError_t ea = cudaMalloc(&bt->d_pair, b_lat + b_tile + b_row + b_node + 2 * b_fb + b_F);
+    const size_t image = b_lat + b_tile + b_row + b_node;
+    const cudaError_t ea = pair_memory_alloc(bt->pair, image + 2 * b_fb + b_F, image);
     if (ea != cudaSuccess) {
-        cudaGetLastError();
-        bt->d_pair = nullptr;
-        return bfail(bt, ea == cudaErrorMemoryAllocation ? BTDF_ENOMEM : BTDF_ECUDA, "pair tables");
+        bt->pair_nomem = ea == cudaErrorMemoryAllocation;
+        return BTDF_ENOMEM;
     }
-    char* q = (char*)bt->d_pair;
+    char* q = (char*)bt->pair.dev;
     PairLattice* d_lat = (PairLattice*)q;
     int4* d_tile = (int4*)(q += b_lat);
     int* d_row = (int*)(q += b_tile);
@@ -400,15 +404,17 @@ int ensure_pair_tables(btdf_batch* bt) try {
     bt->d_F1 = (float2*)(q += b_fb);
     for (int c = 0; c < bt->n; c++)
         if (bt->nmark > 0 && !bt->band_keys[c].empty()) lat[c].strip_row = d_row + row0[c];
-    cudaStream_t st = bt->stream;
-    BCK(cudaMemcpyAsync(d_lat, lat.data(), sizeof(PairLattice) * bt->n, cudaMemcpyHostToDevice, st));
-    BCK(cudaMemcpyAsync(d_tile, tiles.data(), sizeof(int4) * tiles.size(), cudaMemcpyHostToDevice, st));
-    if (!strip_row.empty())
-        BCK(cudaMemcpyAsync(d_row, strip_row.data(), sizeof(int) * strip_row.size(), cudaMemcpyHostToDevice, st));
-    if (!nodes.empty())
-        BCK(cudaMemcpyAsync(d_node, nodes.data(), sizeof(int4) * nodes.size(), cudaMemcpyHostToDevice, st));
-    BCK(cudaMemsetAsync(d_fb1, 0, 2 * b_fb + b_F, st));   // band nodes without terms keep a zero force
-    BCK(cudaStreamSynchronize(st));
+    char* const pin = (char*)bt->pair.pin;
+    memcpy(pin, lat.data(), sizeof(PairLattice) * bt->n);
+    memcpy(pin + b_lat, tiles.data(), sizeof(int4) * tiles.size());
+    if (!strip_row.empty()) memcpy(pin + b_lat + b_tile, strip_row.data(), sizeof(int) * strip_row.size());
+    if (!nodes.empty()) memcpy(pin + b_lat + b_tile + b_row, nodes.data(), sizeof(int4) * nodes.size());
+    // band nodes without terms keep a zero force
+    const cudaError_t eu = pair_memory_upload(bt->pair, image + 2 * b_fb + b_F, image, bt->stream);
+    if (eu != cudaSuccess) {
+        pair_memory_free(bt->pair);
+        return bfail(bt, BTDF_ECUDA, std::string("uploading the pair tables: ") + cudaGetErrorString(eu));
+    }
     PairForces f{};
     f.F1 = bt->d_F1;
     f.nodes = d_node;
@@ -425,7 +431,8 @@ int ensure_pair_tables(btdf_batch* bt) try {
     bt->pb = b;
     return BTDF_OK;
 } catch (const std::bad_alloc&) {
-    return bfail(bt, BTDF_ENOMEM, "pair tables do not fit");
+    bt->pair_nomem = true;
+    return BTDF_ENOMEM;
 }
 
 // Pairs of steps unless a launch shape was chosen: with every support inside.
@@ -847,16 +854,21 @@ int btdf_batch_step(btdf_batch* bt, int64_t nsteps) {
     if (nsteps < 0) return bfail(bt, BTDF_EINVAL, "nsteps < 0");
     for (int c = 0; c < bt->n; c++)
         if (!bt->has_fields[c]) return bfail(bt, BTDF_ESTATE, "every lattice needs btdf_batch_init_fields");
-    int64_t i = 0;
+    int64_t i = 0;   // steps issued so far
+    // what has been issued counts, also where the rest cannot be
+    auto stop = [&](int rc) {
+        bt->steps += i;
+        return rc;
+    };
     bool pairs = nsteps - (bt->poststream ? 1 : 0) >= 2 && pairs_allowed(bt);
     const bool captured = pairs && stream_captures(bt->stream);
-    if (pairs && !bt->d_pair) {
+    if (pairs && !bt->pair.dev) {
         // no tables while the caller captures the stream; single steps need none
         if (captured) {
             pairs = false;
         } else {
             const int rc = ensure_pair_tables(bt);
-            if (rc == BTDF_ENOMEM) pairs = false, bt->pair_nomem = true;
+            if (rc == BTDF_ENOMEM) pairs = false;
             else if (rc != BTDF_OK) return rc;
         }
     }
@@ -869,20 +881,21 @@ int btdf_batch_step(btdf_batch* bt, int64_t nsteps) {
     }
     while (nsteps - i >= kBatchGraphSteps) {
         const int rc = ensure_graph(bt, bt->cur, pairs);
-        if (rc != BTDF_OK) return rc;
-        BCK(cudaGraphLaunch(bt->gexec[bt->cur], bt->stream));
+        if (rc != BTDF_OK) return stop(rc);
+        const cudaError_t e = cudaGraphLaunch(bt->gexec[bt->cur], bt->stream);
+        if (e != cudaSuccess)
+            return stop(bfail(bt, BTDF_ECUDA, std::string("cudaGraphLaunch: ") + cudaGetErrorString(e)));
         i += kBatchGraphSteps;
     }
     int64_t npairs = pairs ? pairs_of(nsteps - i, captured) : 0;
     while (i < nsteps) {
         const bool two = npairs-- > 0;
         const int rc = two ? enqueue_pair(bt, bt->stream, bt->cur) : enqueue(bt, bt->stream, true, bt->cur);
-        if (rc != BTDF_OK) return rc;
+        if (rc != BTDF_OK) return stop(rc);
         bt->cur = 1 - bt->cur;
         i += two ? 2 : 1;
     }
-    bt->steps += nsteps;
-    return BTDF_OK;
+    return stop(BTDF_OK);
 }
 
 int btdf_batch_sync(btdf_batch* bt) {

@@ -202,4 +202,35 @@ void build_pair_tables(int nx, int ny, int nseg, bool px, int npl, int nstrip, c
     }
 }
 
+cudaError_t pair_memory_alloc(PairMemory& m, size_t dev_bytes, size_t pin_bytes) {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaError_t e = cudaThreadExchangeStreamCaptureMode(&mode);
+    if (e == cudaSuccess) {
+        e = cudaMalloc(&m.dev, dev_bytes);
+        if (e == cudaSuccess) e = cudaMallocHost(&m.pin, pin_bytes);
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&m.uploaded, cudaEventDisableTiming);
+        if (e != cudaSuccess) pair_memory_free(m);
+        cudaThreadExchangeStreamCaptureMode(&mode);
+    }
+    if (e != cudaSuccess) cudaGetLastError();
+    return e;
+}
+
+cudaError_t pair_memory_upload(PairMemory& m, size_t dev_bytes, size_t pin_bytes, cudaStream_t st) {
+    cudaError_t e = cudaMemcpyAsync(m.dev, m.pin, pin_bytes, cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync((char*)m.dev + pin_bytes, 0, dev_bytes - pin_bytes, st);
+    if (e == cudaSuccess) e = cudaEventRecord(m.uploaded, st);
+    return e;
+}
+
+void pair_memory_free(PairMemory& m) {
+    if (m.uploaded) {
+        cudaEventSynchronize(m.uploaded);
+        cudaEventDestroy(m.uploaded);
+    }
+    if (m.pin) cudaFreeHost(m.pin);
+    if (m.dev) cudaFree(m.dev);
+    m = PairMemory{};
+}
+
 }  // namespace btdf
