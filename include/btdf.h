@@ -197,8 +197,9 @@ int btdf_move_markers(btdf_ctx *ctx, int32_t body, const double *X, const double
  * stream: the call never waits for the stream.  Requires btdf_init_fields or
  * btdf_load_state first (ESTATE).  The call in which steps first go in pairs
  * (btdf_tune, variant 0) after markers were added or moved builds their tables on
- * the host (0.1 ms with one body, a few ms with hundreds) and allocates device and
- * page-locked memory for them; where that cannot be had the steps are taken
+ * the host (some 0.03 ms with one body, a few ms with hundreds; so it waits until
+ * the steps on the same markers pay for them) and allocates device memory, for
+ * large ones also page-locked memory; where that cannot be had the steps are taken
  * singly.  After an error the step counter holds the steps that were issued.
  * A call that the caller captures into a CUDA graph keeps its parity: an even
  * number of steps ends in the population buffer it began with, so that replays

@@ -85,6 +85,8 @@ namespace {
 constexpr int kGraphSteps = 64;          // steps per replayed CUDA graph (a multiple of 4: an even number of pairs)
 constexpr int kFullGrid = 1 << 30;       // grid cap meaning "one row segment per warp"
 constexpr int kSchedWords = 3;           // device counters: the two of LatticeParams.sched, pair_kernel's
+constexpr double kLeadNodes = 1 << 23;   // from here on, kLeadSteps single steps run while tables are built
+constexpr int kLeadSteps = 6;
 constexpr int kStageSlots = 4;           // pinned staging slots for marker velocities
 constexpr uint64_t kStateMagic = 0x3230465444544242ull;   // "BBTDTF02"
 
@@ -557,8 +559,8 @@ int ensure_pair_tables(btdf_ctx* ctx) try {
         ctx->pair_nomem = ea == cudaErrorMemoryAllocation;
         return BTDF_ENOMEM;
     }
-    memcpy((char*)ctx->pair.pin + o_srow, strip_row.data(), sizeof(int) * strip_row.size());
-    if (!bnodes.empty()) memcpy((char*)ctx->pair.pin + o_bn, bnodes.data(), sizeof(int4) * bnodes.size());
+    memcpy((char*)ctx->pair.image + o_srow, strip_row.data(), sizeof(int) * strip_row.size());
+    if (!bnodes.empty()) memcpy((char*)ctx->pair.image + o_bn, bnodes.data(), sizeof(int4) * bnodes.size());
     const cudaError_t eu = pair_memory_upload(ctx->pair, A.size, o_fb0, ctx->stream);
     if (eu != cudaSuccess) {
         pair_memory_free(ctx->pair);
@@ -576,6 +578,22 @@ int ensure_pair_tables(btdf_ctx* ctx) try {
 } catch (const std::bad_alloc&) {
     ctx->pair_nomem = true;
     return BTDF_ENOMEM;
+}
+
+// Steps on the same markers that pay for the tables.  They cost the host, in us,
+// about 20 and 0.14 a marker (50 markers 21, 126 38, 3780 590, 12 600 1690).  A step
+// of a pair saves, in us, FP32 / FP16: 160 x 80 1.8 / 3.7, 800 x 400 2.0 / 3.1,
+// 1600 x 800 3.3 / 2.2 (with 3780 markers 10 / 11), 2048 x 2048 16 / 6.5, 4096 x
+// 2048 32 / 7.0 (with 21 546 markers 23 / 12), 8192 x 4096 134 / 14.  So 2048 x 2048
+// FP32 asks for 3 steps with one body and 107 with 100; one rule by size and storage (16 from 2^22 nodes in FP32,
+// 256 in 16 bits) built the latter's tables for 33 steps, 5.6 ms instead of 3.4, and
+// left a 4096 x 1024 FP16 lattice with one body on single steps for 256 instead of 9.
+int64_t pair_worth(const btdf_ctx* ctx) {
+    const double n = (double)ctx->cfg.nx * ctx->cfg.ny, m = ctx->nmark;
+    const bool f32 = ctx->cfg.storage == kStoreF32;
+    const double saved = n >= (double)(1 << 22) ? (f32 ? 4e-6 * n : 3.0 + 0.33e-6 * n + 0.25e-3 * m)
+                                                : (f32 ? 1.5 + 1.3e-6 * n : 3.0) + 1.8e-3 * m;
+    return (n >= kLeadNodes ? kLeadSteps : 0) + 1 + (int64_t)((20.0 + 0.14 * m) / saved);
 }
 
 // Issues the kernels of two pulling time steps reading buffer `cur`; the state
@@ -1317,14 +1335,9 @@ int btdf_step(btdf_ctx* ctx, int64_t nsteps) {
     };
     bool pairs = nsteps - (ctx->poststream ? 1 : 0) >= 2 && pairs_allowed(ctx);
     if (pairs && ctx->nmark > 0 && !ctx->pair.dev) {
-        // Building the tables takes the host 0.1-0.3 ms with one body (2-3 ms with
-        // hundreds); a pair saves 2-6 us a step on small lattices, and on large ones
-        // 100 in FP32 but 11 in 16-bit storage.  So bodies that move every few steps
-        // keep single steps, and the tables are built once the markers have been used
-        // for about as many steps as pay for them.
-        const bool large = (long long)ctx->cfg.nx * ctx->cfg.ny >= (1ll << 22);
-        const int64_t worth = !large ? 64 : ctx->cfg.storage == kStoreF32 ? 16 : 256;
-        if (ctx->marker_steps + nsteps < worth) pairs = false;
+        // Bodies that move every few steps keep single steps: the tables are built
+        // once the markers are used for as many steps as pay for them.
+        if (ctx->marker_steps + nsteps < pair_worth(ctx)) pairs = false;
     }
     const bool captured = pairs && stream_captures(ctx->stream);
     // the tables cannot be built while the caller captures the stream
@@ -1337,11 +1350,10 @@ int btdf_step(btdf_ctx* ctx, int64_t nsteps) {
         i = 1;
     }
     if (pairs) {
-        // The tables of the pair kernels take the host 2-3 ms with hundreds of
-        // bodies: on a large lattice a few single steps keep the device busy
-        // meanwhile.
-        if (ctx->nmark > 0 && !ctx->pair.dev && (long long)ctx->cfg.nx * ctx->cfg.ny >= (1ll << 23))
-            for (int k = 0; k < 6 && i < nsteps; k++, i++) {
+        // The tables take the host up to 3 ms: on a large lattice a few single steps
+        // keep the device busy meanwhile.
+        if (ctx->nmark > 0 && !ctx->pair.dev && (double)ctx->cfg.nx * ctx->cfg.ny >= kLeadNodes)
+            for (int k = 0; k < kLeadSteps && i < nsteps; k++, i++) {
                 const int rc = enqueue_step(ctx, ctx->stream, true, ctx->cur, false);
                 if (rc != BTDF_OK) return stop(rc);
                 ctx->cur = 1 - ctx->cur;

@@ -404,11 +404,11 @@ int ensure_pair_tables(btdf_batch* bt) try {
     bt->d_F1 = (float2*)(q += b_fb);
     for (int c = 0; c < bt->n; c++)
         if (bt->nmark > 0 && !bt->band_keys[c].empty()) lat[c].strip_row = d_row + row0[c];
-    char* const pin = (char*)bt->pair.pin;
-    memcpy(pin, lat.data(), sizeof(PairLattice) * bt->n);
-    memcpy(pin + b_lat, tiles.data(), sizeof(int4) * tiles.size());
-    if (!strip_row.empty()) memcpy(pin + b_lat + b_tile, strip_row.data(), sizeof(int) * strip_row.size());
-    if (!nodes.empty()) memcpy(pin + b_lat + b_tile + b_row, nodes.data(), sizeof(int4) * nodes.size());
+    char* const im = (char*)bt->pair.image;
+    memcpy(im, lat.data(), sizeof(PairLattice) * bt->n);
+    memcpy(im + b_lat, tiles.data(), sizeof(int4) * tiles.size());
+    if (!strip_row.empty()) memcpy(im + b_lat + b_tile, strip_row.data(), sizeof(int) * strip_row.size());
+    if (!nodes.empty()) memcpy(im + b_lat + b_tile + b_row, nodes.data(), sizeof(int4) * nodes.size());
     // band nodes without terms keep a zero force
     const cudaError_t eu = pair_memory_upload(bt->pair, image + 2 * b_fb + b_F, image, bt->stream);
     if (eu != cudaSuccess) {
@@ -433,6 +433,18 @@ int ensure_pair_tables(btdf_batch* bt) try {
 } catch (const std::bad_alloc&) {
     bt->pair_nomem = true;
     return BTDF_ENOMEM;
+}
+
+// As pair_worth of one lattice.  The tables cost the host about 0.23 us a marker
+// (190 markers 41 us, 1613 364, 4778 1083); a step of a pair saves, in us,
+// FP32 / FP16: 4 lattices of 16 k nodes 6.6 / 6.8, 24 of 57 k 15 / 11, 64 of 210 k
+// 56 / 45, 128 of 203 k 80 / 53.  Built for the first two steps instead, a first call
+// of 3 steps took 472 us against 118 singly on the 24, 1410 against 606 on the 64.
+int64_t pair_worth(const btdf_batch* bt) {
+    double n = 0.0;
+    for (const btdf_config& k : bt->cfg) n += (double)k.nx * k.ny;
+    const double m = bt->nmark;
+    return (int64_t)((10.0 + 0.23 * m) / (6.0 + (bt->storage == kStoreF32 ? 3.2e-6 : 2.2e-6) * n + 2e-3 * m));
 }
 
 // Pairs of steps unless a launch shape was chosen: with every support inside.
@@ -861,23 +873,28 @@ int btdf_batch_step(btdf_batch* bt, int64_t nsteps) {
         return rc;
     };
     bool pairs = nsteps - (bt->poststream ? 1 : 0) >= 2 && pairs_allowed(bt);
+    if (pairs && !bt->pair.dev && bt->steps + nsteps < pair_worth(bt)) pairs = false;
     const bool captured = pairs && stream_captures(bt->stream);
-    if (pairs && !bt->pair.dev) {
-        // no tables while the caller captures the stream; single steps need none
-        if (captured) {
-            pairs = false;
-        } else {
-            const int rc = ensure_pair_tables(bt);
-            if (rc == BTDF_ENOMEM) pairs = false;
-            else if (rc != BTDF_OK) return rc;
-        }
-    }
+    if (captured && !bt->pair.dev) pairs = false;   // no tables while the caller captures the stream
     if (nsteps > 0 && bt->poststream) {
         const int rc = enqueue(bt, bt->stream, false, bt->cur);
         if (rc != BTDF_OK) return rc;
         bt->cur = 1 - bt->cur;
         bt->poststream = false;
         i = 1;
+    }
+    if (pairs) {
+        // the host builds the tables while the device takes the step before, on
+        // large batches a few more
+        if (!bt->pair.dev && bt->total >= 9ull << 22)
+            for (int k = 0; k < 6 && i < nsteps; k++, i++) {
+                const int rc = enqueue(bt, bt->stream, true, bt->cur);
+                if (rc != BTDF_OK) return stop(rc);
+                bt->cur = 1 - bt->cur;
+            }
+        const int rc = ensure_pair_tables(bt);
+        if (rc == BTDF_ENOMEM) pairs = false;   // single steps need no tables
+        else if (rc != BTDF_OK) return stop(rc);
     }
     while (nsteps - i >= kBatchGraphSteps) {
         const int rc = ensure_graph(bt, bt->cur, pairs);

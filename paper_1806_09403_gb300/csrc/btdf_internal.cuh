@@ -275,19 +275,23 @@ cudaError_t launch_ib_pair_batch(int storage, int width, const void* g, const La
 // Rows of the pair kernel's tiles.
 int pair_tile_rows(int npl);
 
-// Memory of the pair kernels' tables: `dev`, and the page-locked image of the part
-// of it that the host builds.  A step call allocates both and enqueues the upload,
-// without waiting for the stream; the image lives as long as the tables.
+// Memory of the pair kernels' tables: `dev`, and the host's image of the part of it
+// that the host builds.  A step call allocates both and enqueues the upload,
+// without waiting for the stream; the image lives as long as the tables.  Up to
+// kPairChunks copies of kPairChunk bytes, which never wait for the stream, the image
+// is pageable; a larger one is page-locked, which takes the call 0.1 ms more.
+constexpr size_t kPairChunk = 64 << 10, kPairChunks = 16;
 struct PairMemory {
-    void *dev = nullptr, *pin = nullptr;
+    void *dev = nullptr, *image = nullptr;
+    bool pinned = false;
     cudaEvent_t uploaded = nullptr;
 };
 // Allocates, also while some thread captures a stream of its own (a stream's
 // capture has nothing to do with this memory).  Leaves `m` empty and no CUDA error
 // behind where it fails.
-cudaError_t pair_memory_alloc(PairMemory& m, size_t dev_bytes, size_t pin_bytes);
+cudaError_t pair_memory_alloc(PairMemory& m, size_t dev_bytes, size_t image_bytes);
 // Enqueues the upload of the image, and zeros behind it.
-cudaError_t pair_memory_upload(PairMemory& m, size_t dev_bytes, size_t pin_bytes, cudaStream_t st);
+cudaError_t pair_memory_upload(PairMemory& m, size_t dev_bytes, size_t image_bytes, cudaStream_t st);
 void pair_memory_free(PairMemory& m);
 void build_pair_tables(int nx, int ny, int nseg, bool px, int npl, int nstrip, const std::vector<int>& keys,
                        const std::vector<int>& seg_ptr, int term0, std::vector<int>& strip_row,

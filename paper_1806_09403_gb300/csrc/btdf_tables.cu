@@ -6,6 +6,7 @@
 #include "btdf_internal.cuh"
 
 #include <algorithm>
+#include <cstdlib>
 #include <cmath>
 
 namespace btdf {
@@ -202,12 +203,16 @@ void build_pair_tables(int nx, int ny, int nseg, bool px, int npl, int nstrip, c
     }
 }
 
-cudaError_t pair_memory_alloc(PairMemory& m, size_t dev_bytes, size_t pin_bytes) {
+cudaError_t pair_memory_alloc(PairMemory& m, size_t dev_bytes, size_t image_bytes) {
     cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
     cudaError_t e = cudaThreadExchangeStreamCaptureMode(&mode);
     if (e == cudaSuccess) {
         e = cudaMalloc(&m.dev, dev_bytes);
-        if (e == cudaSuccess) e = cudaMallocHost(&m.pin, pin_bytes);
+        m.pinned = image_bytes > kPairChunk * kPairChunks;
+        if (e == cudaSuccess) {
+            if (m.pinned) e = cudaMallocHost(&m.image, image_bytes);
+            else if ((m.image = std::malloc(image_bytes)) == nullptr) e = cudaErrorMemoryAllocation;
+        }
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&m.uploaded, cudaEventDisableTiming);
         if (e != cudaSuccess) pair_memory_free(m);
         cudaThreadExchangeStreamCaptureMode(&mode);
@@ -216,9 +221,13 @@ cudaError_t pair_memory_alloc(PairMemory& m, size_t dev_bytes, size_t pin_bytes)
     return e;
 }
 
-cudaError_t pair_memory_upload(PairMemory& m, size_t dev_bytes, size_t pin_bytes, cudaStream_t st) {
-    cudaError_t e = cudaMemcpyAsync(m.dev, m.pin, pin_bytes, cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync((char*)m.dev + pin_bytes, 0, dev_bytes - pin_bytes, st);
+cudaError_t pair_memory_upload(PairMemory& m, size_t dev_bytes, size_t image_bytes, cudaStream_t st) {
+    cudaError_t e = cudaSuccess;
+    const size_t step = m.pinned ? image_bytes : kPairChunk;
+    for (size_t o = 0; o < image_bytes && e == cudaSuccess; o += step)
+        e = cudaMemcpyAsync((char*)m.dev + o, (const char*)m.image + o, std::min(step, image_bytes - o),
+                            cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync((char*)m.dev + image_bytes, 0, dev_bytes - image_bytes, st);
     if (e == cudaSuccess) e = cudaEventRecord(m.uploaded, st);
     return e;
 }
@@ -228,7 +237,7 @@ void pair_memory_free(PairMemory& m) {
         cudaEventSynchronize(m.uploaded);
         cudaEventDestroy(m.uploaded);
     }
-    if (m.pin) cudaFreeHost(m.pin);
+    if (m.image) m.pinned ? (void)cudaFreeHost(m.image) : std::free(m.image);
     if (m.dev) cudaFree(m.dev);
     m = PairMemory{};
 }
