@@ -1029,19 +1029,35 @@ __global__ void init_kernel(T* g, LatticeParams p, const double* rho, const doub
     }
 }
 
-// One thread per node, consecutive lanes along x.  The nine loads of a node go
+// One thread per node in the order of dst, so that narrow lattices fill their
+// blocks too.  The nine loads of a node go
 // out together (gather_node); through read_node's out-of-line pull with its
 // stack array the populations of 8192 x 4096 took 884 us to read in FP32; the pass
-// that steps 50 times and reads them went from 12.66 to 12.11 ms.
-template <typename T>
-__global__ void __launch_bounds__(kThreads) read_field_kernel(const T* __restrict__ g, const __grid_constant__ LatticeParams p,
-                                                              int pull, int kind, int row_blocks, float* __restrict__ dst) {
-    const int y = (int)blockIdx.x / row_blocks;
-    const int x = ((int)blockIdx.x - y * row_blocks) * kThreads + (int)threadIdx.x;
-    if (x >= p.nx) return;
-    const long long nn = (long long)p.nx * p.ny, n = (long long)y * p.nx + x;
+// that steps 50 times and reads them went from 12.66 to 12.11 ms.  With blocks for
+// every row, reading 2^22 nodes 4 wide took 1472 us (FP16 1567), now 225 (139); 64
+// wide 157 (188), now 85 (81).
+// kFold: the populations of inlet and outlet nodes come from the node beside them,
+// so its loads go out with the rest of the warp's and the rule follows; on its own
+// path the row ends' loads double a narrow lattice's time (64 wide 136 us).
+template <typename T, bool kFold>
+__global__ void __launch_bounds__(kThreads, 8) read_field_kernel(const T* __restrict__ g, const __grid_constant__ LatticeParams p,
+                                                              int pull, int kind, float* __restrict__ dst) {
+    const unsigned n = blockIdx.x * kThreads + threadIdx.x;   // a lattice has fewer than 2^32 / 9 nodes
+    const long long nn = (long long)p.nx * p.ny;
+    if (n >= (unsigned)nn) return;
+    const int y = (int)(n / (unsigned)p.nx), x = (int)(n - (unsigned)y * (unsigned)p.nx);
     float d[9];
-    gather_node<T>(g, p, pull != 0, x, y, d);
+    gather_node<T>(g, p, pull != 0, kFold ? min(max(x, 1), p.nx - 2) : x, y, d);
+    if (kFold && x == 0) {
+        float f1[9];
+#pragma unroll
+        for (int a = 0; a < 9; a++) f1[a] = d[a];
+        inlet_from(f1, p, d);
+    }
+    if (kFold && x == p.nx - 1 && p.outlet != nullptr) {
+#pragma unroll
+        for (int a = 0; a < 9; a++) d[a] = __fmaf_rn(p.uc_new, d[a], __fmul_rn(p.uc_old, p.outlet[a * p.ny + y]));
+    }
     if (kind == 3) {
 #pragma unroll
         for (int a = 0; a < 9; a++)
@@ -1482,19 +1498,21 @@ cudaError_t launch_init_equilibrium(int storage, void* g, const LatticeParams& p
 
 cudaError_t launch_read_field(int storage, bool pull, const void* g, const LatticeParams& p, int kind,
                               float* dst, cudaStream_t st) {
-    const int rb = (p.nx + kThreads - 1) / kThreads;
-    const unsigned nb = (unsigned)rb * (unsigned)p.ny;
+    const unsigned nb = blocks_for((long long)p.nx * p.ny);
     const int pl = pull ? 1 : 0;
+    // from 4096 columns on too few warps hold a row end for the folded form to pay:
+    // 8192 x 4096 FP32 443 us against 438, the density 333 against 317
+    const bool fold = pull && p.bcx == kBcxInout && p.box == nullptr && p.nx < 4096;
     switch (storage) {
     case kStoreF32:
-        read_field_kernel<float><<<nb, kThreads, 0, st>>>((const float*)g, p, pl, kind, rb, dst);
+        (fold ? read_field_kernel<float, true> : read_field_kernel<float, false>)<<<nb, kThreads, 0, st>>>((const float*)g, p, pl, kind, dst);
         break;
     case kStoreF16:
-        read_field_kernel<__half><<<nb, kThreads, 0, st>>>((const __half*)g, p, pl, kind, rb, dst);
+        (fold ? read_field_kernel<__half, true> : read_field_kernel<__half, false>)<<<nb, kThreads, 0, st>>>((const __half*)g, p, pl, kind, dst);
         break;
     case kStoreBF16:
-        read_field_kernel<__nv_bfloat16>
-            <<<nb, kThreads, 0, st>>>((const __nv_bfloat16*)g, p, pl, kind, rb, dst);
+        (fold ? read_field_kernel<__nv_bfloat16, true> : read_field_kernel<__nv_bfloat16, false>)
+            <<<nb, kThreads, 0, st>>>((const __nv_bfloat16*)g, p, pl, kind, dst);
         break;
     default: return cudaErrorInvalidValue;
     }

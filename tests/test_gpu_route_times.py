@@ -1,5 +1,5 @@
 """The kernels that the library chooses by itself are not slower than others it
-has for the same work.  Both sides are timed in turn in one process, the lowest
+has for the same work, and right at the edges of their blocks.  Both sides are timed in turn in one process, the lowest
 of several runs each; the margins are several times what such runs differ."""
 import numpy as np
 import pytest
@@ -64,3 +64,33 @@ def test_automatic_steps_are_not_slower_than_single_ones(nx, ny, storage, bcx, s
     lats[1].tune(single)
     auto, one = lowest([lambda x=x: x.step(512) for x in lats])
     assert auto < 1.04 * one, (auto, one)
+
+
+def test_reading_a_narrow_lattice():
+    """Lattices 4 nodes wide are padded to 32 columns, so reading one costs some
+    three times what a wide one of as many nodes does (17 times where every row has
+    blocks of its own)."""
+    lats = [lattice(4, 1 << 20, B.BTDF_F32), lattice(2048, 2048, B.BTDF_F32)]
+    out = torch.empty(9 << 22, device="cuda")
+    for x in lats:
+        x.step(2)
+    narrow, wide = lowest([lambda x=x: x.field_to_device(B.FIELD_POPS, out.data_ptr()) for x in lats])
+    assert narrow < 8 * wide, (narrow, wide)
+
+
+@pytest.mark.parametrize("storage,half_ulp", [(B.BTDF_F32, 2.0 ** -24), (B.BTDF_F16DEV, 2.0 ** -12),
+                                              (B.BTDF_BF16DEV, 2.0 ** -9)])
+@pytest.mark.parametrize("nx,ny", [(4, 4), (5, 61), (16, 65), (255, 7), (256, 4), (257, 9)])
+def test_reading_fields_at_block_edges(nx, ny, storage, half_ulp):
+    """Rows that end within a block of the read-out.  A new lattice's moments are
+    its initial fields up to the rounding of nine stored deviations of at most
+    0.1, and of the read-out's own sums in FP32."""
+    lat = lattice(nx, ny, storage)
+    rng = np.random.default_rng(nx * ny)
+    rho, ux, uy = (c + rng.uniform(-0.02, 0.02, (ny, nx)) for c in (1.0, 0.05, 0.0))
+    lat.init_fields(rho, ux, uy)
+    tol = 2 * 9 * 0.1 * half_ulp + 1e-6
+    for want, kind in ((rho, B.FIELD_RHO), (ux, B.FIELD_UX), (uy, B.FIELD_UY)):
+        assert np.abs(lat.field(kind) - want).max() < tol
+    pops = lat.field(B.FIELD_POPS)
+    assert np.abs(pops.sum(0) - rho).max() < tol
