@@ -460,7 +460,7 @@ __device__ __forceinline__ void pair_tile(const T* __restrict__ gin, T* __restri
             for (int i = 0; i < NP; i++) f[a][i] = u.get(i);
         }
         if ((ends && !perx) || (noslip && !inner))
-            pair_boundaries<T, NPL>(f, p, x0, rr, ends, p.outlet, own && j > 0 && j <= TH);
+            pair_boundaries<T, NPL>(f, p, x0, rr, ends, p.outlet, own && j > 0 && j <= TH && r < ny);
         T* const trow = tile + j * C::W + NPL * lane;
         P2 Fx[NP] = {}, Fy[NP] = {};
         if (uniform_force || band >= 0) {
