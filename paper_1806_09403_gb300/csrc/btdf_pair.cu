@@ -306,8 +306,9 @@ struct PairTile {
 // of the populations that come back from a bounce-back wall; the inlet node from
 // the node beside it, the outlet node from the node before it, which may be the
 // lane below's last (old: the convective outlet's previous column; keep: write
-// the new one).  Inner nodes take the wall's constant with one rounding, row
-// ends (g; those of a periodic lattice too) with two, as the single steps do.
+// the new one).  As in the single steps, inner nodes take the wall's constant with
+// one rounding, row ends (g; those of a periodic lattice too) with two; in FP16,
+// whose constant is rounded before it is scaled, all nodes take it with two.
 // One population at a time: arrays of the lane's nodes would raise the register
 // count of the whole kernel.
 template <typename T, int NPL>
@@ -336,7 +337,7 @@ __device__ __forceinline__ void pair_boundaries(P2 (&fp)[9][NPL / 2], const Latt
                     g[a][i] = __fadd_rn(f[a][i], add);
                     const int x = x0 + i;
                     const bool end = perx && (x == -1 || x == 0 || x == nx - 1 || x == nx);
-                    f[a][i] = end ? g[a][i] : __fmaf_rn(w, p.eur[a], f[a][i]);
+                    f[a][i] = end || up != 1.0f ? g[a][i] : __fmaf_rn(w, p.eur[a], f[a][i]);
                 }
             }
     }
@@ -671,13 +672,13 @@ __device__ __forceinline__ void ib_pair_marker(const T* __restrict__ g, const La
 #pragma unroll
         for (int a = 0; a < 9; a++) f[k][a][0] = d[a] * Raw<T>::kScale;
         // the LBM kernels add a bounce-back wall's constant with one rounding
-        // on inner columns
-        if (p.bcy == kBcyNoslip && (y == 0 || y == p.ny - 1) && x > 0 && x < p.nx - 1) {
+        // on inner columns (not in FP16: pair_boundaries)
+        if (Raw<T>::kScale == 1.0f && p.bcy == kBcyNoslip && (y == 0 || y == p.ny - 1) && x > 0 && x < p.nx - 1) {
 #pragma unroll
             for (int a = 0; a < 9; a++)
                 if ((ey(a) > 0 && y == 0) || (ey(a) < 0 && y == p.ny - 1)) {
                     const float v = Io<T>::ld1(g + p.poff[opposite(a)] + (unsigned)y * p.rs + (unsigned)x);
-                    f[k][a][0] = __fmaf_rn(-6.0f * wt(a), p.eur[a], v) * Raw<T>::kScale;
+                    f[k][a][0] = __fmaf_rn(-6.0f * wt(a), p.eur[a], v);
                 }
         }
         const int seg = __ldg(p.seg_index + y * p.nseg + x / kSeg);
