@@ -515,14 +515,21 @@ bool pairs_possible(const btdf_ctx* ctx) {
     return !ctx->prof && !ctx->d_box && (ctx->nmark == 0 || (ctx->cfg.nf == 1 && ctx->markers_inside));
 }
 
-// Whether the context takes them: with the automatic variant (they are the faster
-// form at every size: us a step, singly -> in pairs, with one body: 160 x 80 FP32
-// 6.1 -> 4.9, FP16 8.7 -> 5.6; 800 x 400 7.2 -> 5.9 and 8.4 -> 6.2; 1600 x 800
-// 14.8 -> 11.6 and 13.3 -> 11.1; 160 x 80 without bodies 3.8 -> 2.0), or after the
-// autotuner found them so.
+// Whether the context takes them: with the automatic variant where its strips suit
+// the lattice (pairs_pay; there they are the faster form at every size.  us a step,
+// singly -> in pairs, with one body and the 3-point delta: 160 x 80 FP32 6.1 -> 4.7,
+// FP16 8.7 -> 5.3; 800 x 400 7.2 -> 5.7 and 8.4 -> 5.4; 1600 x 800 14.8 -> 11.5 and
+// 13.3 -> 10.7; with the 4-point cosine 160 x 80 6.1 -> 6.0 and 8.8 -> 6.4, 800 x 400
+// 7.2 -> 6.6 and 8.4 -> 6.7; 160 x 80 without bodies 3.7 -> 2.1), or after the autotuner
+// found them so.
 bool pairs_allowed(const btdf_ctx* ctx) {
     if (!pairs_possible(ctx)) return false;
-    return ctx->variant == kVarAuto && ctx->grid_override == 0 ? true : ctx->pairs_tuned;
+    if (ctx->variant != kVarAuto || ctx->grid_override != 0) return ctx->pairs_tuned;
+    const int v = auto_variant(ctx), nx = ctx->cfg.nx;
+    const int bcx = ctx->cfg.bc_x == BTDF_BCX_CONVECTIVE ? kBcxInout : ctx->cfg.bc_x;
+    const int npl = pair_npl(ctx->cfg.storage, bcx, nx, ctx->cfg.ny);
+    return pairs_pay(ctx->cfg.storage, ctx->nmark > 0, (double)nx * ctx->cfg.ny, pair_columns(nx, npl),
+                     single_columns(ctx->nxp, v == kVarReg2 ? 2 : 4));
 }
 
 // Tables of the pair kernels for the current markers, built by the host and

@@ -350,11 +350,16 @@ int rebuild(btdf_batch* bt) {
 int ensure_pair_tables(btdf_batch* bt) try {
     if (bt->pair.dev) return BTDF_OK;
     if (bt->pair_nomem) return BTDF_ENOMEM;
-    long long nodes_all = 0;
-    int npl = 2;
-    for (int c = 0; c < bt->n; c++) nodes_all += (long long)bt->cfg[c].nx * bt->cfg[c].ny;
-    for (int c = 0; c < bt->n; c++)
-        if (nodes_all >= (1ll << 22) || pair_npl(bt->storage, bt->cfg[c].bc_x, bt->cfg[c].nx, bt->cfg[c].ny) == 4) npl = 4;
+    // nodes per lane: pair_npl's rule on the sums over the lattices
+    double nodes_all = 0.0, c2 = 0.0, c4 = 0.0;
+    int npl = bt->storage != kStoreF32 ? 4 : 2;
+    for (const btdf_config& k : bt->cfg) {
+        nodes_all += (double)k.nx * k.ny;
+        c2 += (double)pair_columns(k.nx, 2) * k.ny;
+        c4 += (double)pair_columns(k.nx, 4) * k.ny;
+        if (pair_needs_4(k.bc_x, k.nx)) npl = 4;
+    }
+    if (nodes_all >= (double)(1 << 22) && pair_wide(c2, c4)) npl = 4;
     long long bands = 0;   // slots of the spread arrays are ints, as for one lattice
     for (int c = 0; c < bt->n && bt->nmark > 0; c++)
         bands += (long long)bt->band_keys[c].size() + bt->cfg[c].ny;

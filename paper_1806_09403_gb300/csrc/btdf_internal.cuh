@@ -244,9 +244,22 @@ struct PairForces {
     int nstrip, npl;           // strips, nodes per lane
     unsigned kin[9];           // element offset of population a's source row from the row before
 };
-// Nodes per lane of the pair kernel for a lattice, and its strips.
-int pair_npl(int storage, int bcx, int nx, int ny);
+// Strips of the pair kernel, and the columns that its lanes and those of the single
+// steps' kernels go through in a row.
 inline int pair_strips(int nx, int npl) { return (nx + pair_own(npl) - 1) / pair_own(npl); }
+inline int pair_columns(int nx, int npl) { return pair_strips(nx, npl) * 32 * npl; }
+inline int single_columns(int nxp, int npl) { return (nxp + 32 * npl - 1) / (32 * npl) * 32 * npl; }
+// The outlet column takes its second step from the column before it, which a halo
+// of two nodes does not cover where nx - 1 starts a strip.
+inline bool pair_needs_4(int bcx, int nx) { return bcx == kBcxInout && (nx - 1) % pair_own(2) == 0; }
+// Nodes per lane of the pair kernel for a lattice.
+int pair_npl(int storage, int bcx, int nx, int ny);
+// Whether pairs pay for `nodes` nodes that take them `pair` columns and single steps
+// `single` columns a row.
+bool pairs_pay(int storage, bool bodies, double nodes, double pair, double single);
+// Whether 4 nodes per lane suit lattices that take `c2` columns with 2 and `c4` with
+// 4, streaming from memory.
+inline bool pair_wide(double c2, double c4) { return c4 <= 1.15 * c2; }
 
 // Batched form: a lattice's part of it, its tiles, and the force reductions.
 struct PairLattice {

@@ -828,17 +828,33 @@ cudaError_t ib_pair_t(int width, const void* g, const LatticeParams& p, const Ib
 // Nodes per lane.  FP32 below 2^22 nodes: 2, with 40 warps an SM in tiles of 60 x 6
 // (11.6 us a step at 1600 x 800 against 12.2 with 4); above, where fewer
 // instructions per node count for more, 4, with 27 warps in tiles of 120 x 7
-// (232 us at 8192 x 4096 against 243).  16-bit storage: 4 (1600 x 800 11.1 against
-// 11.4, 8192 x 4096 209 against 239).  Also measured with 4: tiles of 120 x 6 with
+// (232 us at 8192 x 4096 against 243), unless its strips leave many columns unused
+// (128 x 65536: 139 us with 4, 105 with 2, 110 singly). 
+// 16-bit storage: 4 (1600 x 800 11.1 against 11.4, 8192 x 4096 209 against 239).  Also measured with 4: tiles of 120 x 6 with
 // four blocks an SM (FP32 234, FP16 207 at 8192 x 4096, 11.3 at 1600 x 800), 120 x 8
-// with three (240, 209, 11.4).  The outlet column takes its second step from the
-// column before it, which a halo of two nodes does not cover: 4 where nx - 1
-// starts a tile.
+// with three (240, 209, 11.4).
 int pair_npl(int storage, int bcx, int nx, int ny) {
-    if (storage != kStoreF32 || (long long)nx * ny >= (1ll << 22)) return 4;
-    return bcx == kBcxInout && (nx - 1) % pair_own(2) == 0 ? 4 : 2;
+    if (storage != kStoreF32 || pair_needs_4(bcx, nx)) return 4;
+    return (long long)nx * ny >= (1ll << 22) && pair_wide(pair_columns(nx, 2), pair_columns(nx, 4)) ? 4 : 2;
 }
 int pair_tile_rows(int npl) { return npl == 2 ? 6 : 7; }
+
+// A pair halves the launches and the traffic but goes through the columns of whole
+// strips and their halo.  Where those are 1.4 times the single steps' or more (1.5:
+// 122 to 128 columns FP32, 241 to 256 16-bit; 2: 122 to 128 16-bit, 121 FP32) that
+// decides, except on small lattices, where the launches do, and for FP32 beyond L2,
+// where the traffic does.  Pair over single time, without bodies, at 2^16, 2^18, 2^20
+// and 2^22 nodes: 128 columns FP32 0.66, 1.06, 1.01, 0.85, FP16 0.57, 1.12, 1.26, 1.28;
+// 244 FP16 0.56, 0.98, 1.14, 1.15; 121 FP32 -, 1.22, 1.31, 1.14; with one body later:
+// 128 FP16 0.59, 0.78, 1.25.  Below 1.4 pairs were never slower (364 FP16 1.05).
+bool pairs_pay(int storage, bool bodies, double nodes, double pair, double single) {
+    const double waste = pair / single;
+    if (waste < 1.4) return true;
+    auto below = [&](int log2) { return nodes < 0.75 * (1 << log2); };   // 3/4: sizes just below a power count as it
+    if (storage != kStoreF32) return waste < 1.9 ? below(20) : below(bodies ? 19 : 18);
+    if (waste >= 1.9 && single >= 128.0) return below(bodies ? 18 : 17);
+    return below(bodies ? 19 : 18) || nodes >= 1.5 * (1 << 20);
+}
 
 namespace {
 

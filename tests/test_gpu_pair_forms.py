@@ -74,6 +74,24 @@ def test_bounce_back_walls_over_many_nodes(storage, bcx):
         same(a, b, 1)
 
 
+@pytest.mark.parametrize("nx,ny,bcx,bcy", [
+    (128, 32771, W.BCX_INOUT, W.BCY_FREESLIP),       # 2 nodes per lane for its width
+    (2051, 2049, W.BCX_PERIODIC, W.BCY_NOSLIP),      # 4, wrapped columns
+    (2050, 2049, W.BCX_PERIODIC, W.BCY_PERIODIC),
+    (2049, 2051, W.BCX_CONVECTIVE, W.BCY_PERIODIC),
+])
+def test_fp32_beyond_l2(nx, ny, bcx, bcy):
+    wrap = [W.circle_markers(0.3, ny / 3, 12.0, 37)] if bcx == W.BCX_PERIODIC else []
+    a, b = lattices(nx, ny, B.BTDF_F32, bcx, bcy, wrap + [W.circle_markers(nx / 2 + 0.2, ny / 2, 30.0, 94)],
+                    gx=1e-6 if bcx == W.BCX_PERIODIC else 0.0)
+    before = a.device_bytes()
+    for n in (20, 3):
+        a.step(n)
+        b.step(n)
+        same(a, b, n)
+    assert a.device_bytes() > before   # the tables of pairs are there
+
+
 def stable(pair, n):
     """Takes n steps; both sides report a density or force gone astray alike."""
     found = []
