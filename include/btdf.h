@@ -259,7 +259,8 @@ int btdf_state_size(btdf_ctx *ctx, size_t *bytes);
 int btdf_save_state(btdf_ctx *ctx, void *dst, size_t cap, size_t *used);
 int btdf_load_state(btdf_ctx *ctx, const void *src, size_t len);
 
-/* Profiling hooks for benchmarks: while enabled, btdf_step launches every
+/* Profiling hooks for benchmarks: while enabled, btdf_step takes single steps (no
+ * pairs, so not what variant 0 of btdf_tune otherwise runs) and launches every
  * kernel directly (no CUDA graph) between CUDA events on the context stream;
  * btdf_profile_read synchronizes and returns the summed device time of the
  * IB-stage kernels and of the fused collide-stream kernel, and the number of
@@ -275,7 +276,8 @@ int btdf_profile_read(btdf_ctx *ctx, double *ms_ib, double *ms_lbm, int64_t *lau
 /* Variant of the fused collide-stream kernel.  Results do not depend on it.
  *   0 automatic: two steps per pass over the lattice where the call's steps come
  *     in pairs (nf = 1, no box, every marker support inside the lattice and off
- *     the inlet and outlet columns); single steps otherwise: on lattices of at least 2^23 nodes 11 for FP32 and 12 for
+ *     the inlet and outlet columns) and the lattice's width suits them; single
+ *     steps otherwise: on lattices of at least 2^23 nodes 11 for FP32 and 12 for
  *     FP16 / BF16 storage (11 where no tensor maps could be encoded), on
  *     smaller ones 2 for FP32 and 11 for FP16 / BF16 (the autotuner's usual
  *     picks on a GB300)
@@ -309,6 +311,11 @@ int btdf_profile_read(btdf_ctx *ctx, double *ms_ib, double *ms_lbm, int64_t *lau
  * Synchronizes and drops cached CUDA graphs.
  * Errors: EINVAL (unknown variant, TMA variant without tensor maps). */
 int btdf_tune(btdf_ctx *ctx, int32_t variant, int32_t grid_blocks);
+
+/* Whether steps are taken in pairs where they can be (on != 0) or not (0), the
+ * variant of btdf_tune then taking the single steps that remain: the state in which
+ * btdf_autotune leaves a context.  btdf_tune undoes it.  Results do not depend on it. */
+int btdf_tune_pairs(btdf_ctx *ctx, int32_t on);
 
 /* Bound of the TMA-tiled variants' (3-5, 12, 13) per-stage waits, in polls of the
  * stage's mbarrier: polls < 0 restores the default (about a second of
@@ -412,6 +419,8 @@ int btdf_batch_body_lattice(const btdf_batch *b, int32_t body, int32_t *lattice)
  * and off the inlet and outlet columns, else shape 3.  Results do not depend on
  * it. */
 int btdf_batch_tune(btdf_batch *b, int32_t variant);
+/* As btdf_tune_pairs. */
+int btdf_batch_tune_pairs(btdf_batch *b, int32_t on);
 /* As btdf_autotune, over the batch's launch shapes 1..4; ms[0..4], ms[0] being
  * half the time of a pair of steps (-1 where pairs cannot run). */
 int btdf_batch_autotune(btdf_batch *b, int32_t steps, int32_t flush_l2, int32_t *chosen, float *ms);

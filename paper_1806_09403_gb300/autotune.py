@@ -82,26 +82,19 @@ class TuneCache:
 
 def _tune(obj, key: str, cache: TuneCache, run: Callable[[], tuple], apply: Callable[[int], None],
           retune: bool) -> dict:
+    """A hit brings the object into the state in which the autotuner left the one that
+    was timed: its variant for single steps, and pairs of steps if they beat it."""
     hit = None if retune else cache.get(key)
     if hit is not None:
         apply(int(hit["variant"]))
+        if hit.get("pairs"):
+            obj.tune_pairs(True)
         return dict(hit, cached=True)
-    chosen, ms = run()   # the native autotuner leaves the chosen variant applied
-    entry = {"variant": int(chosen), "ms_per_step": {str(k): v for k, v in ms.items()}}
+    chosen, ms = run()
+    entry = {"variant": int(chosen), "ms_per_step": {str(k): v for k, v in ms.items()},
+             "pairs": bool(getattr(obj, "tuned_pairs", False))}
     cache.put(key, entry)
     return dict(entry, cached=False)
-
-
-def _tune_with_pairs(obj, key: str, cache: TuneCache, run, apply, retune: bool) -> dict:
-    """_tune, remembering whether two steps per pass beat the chosen shape: a hit
-    then applies the automatic variant, which takes them."""
-    entry = _tune(obj, key, cache, run, apply, retune)
-    if not entry["cached"]:
-        entry["pairs"] = bool(getattr(obj, "tuned_pairs", False))
-        cache.put(key, {k: v for k, v in entry.items() if k != "cached"})
-    elif entry.get("pairs"):
-        apply(0)
-    return entry
 
 
 def tune_lattice(lat, cache: Optional[TuneCache] = None, steps: int = 20, flush_l2: bool = True,
@@ -110,8 +103,8 @@ def tune_lattice(lat, cache: Optional[TuneCache] = None, steps: int = 20, flush_
     cache miss.  Returns the cache entry with ``cached`` set."""
     cache = cache or TuneCache()
     key = lattice_key(lat, device or device_name())
-    return _tune_with_pairs(lat, key, cache, lambda: lat.autotune(steps, flush_l2),
-                            lambda v: lat.tune(v, 0), retune)
+    return _tune(lat, key, cache, lambda: lat.autotune(steps, flush_l2), lambda v: lat.tune(v, 0),
+                 retune)
 
 
 def tune_batch(bt, cache: Optional[TuneCache] = None, steps: int = 10, flush_l2: bool = False,
@@ -119,4 +112,4 @@ def tune_batch(bt, cache: Optional[TuneCache] = None, steps: int = 10, flush_l2:
     """As tune_lattice for a ``Batch``."""
     cache = cache or TuneCache()
     key = batch_key(bt, device or device_name())
-    return _tune_with_pairs(bt, key, cache, lambda: bt.autotune(steps, flush_l2), bt.tune, retune)
+    return _tune(bt, key, cache, lambda: bt.autotune(steps, flush_l2), bt.tune, retune)

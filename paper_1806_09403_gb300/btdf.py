@@ -39,7 +39,7 @@ EXPORTS = [
     "btdf_batch_last_error", "btdf_set_inflow", "btdf_move_markers", "btdf_adjoint_forward",
     "btdf_adjoint_backward", "btdf_adjoint_release", "btdf_autotune", "btdf_batch_autotune",
     "btdf_read_forces_async", "btdf_add_cylinder", "btdf_set_boundary_velocity",
-    "btdf_set_wait_limit",
+    "btdf_set_wait_limit", "btdf_tune_pairs", "btdf_batch_tune_pairs",
 ]
 STATIC_MAX_MARKERS = 2048
 VARIANT_COUNT = 14          # BTDF_VARIANT_COUNT: variants 0 (automatic) .. 13, see btdf_tune
@@ -107,6 +107,7 @@ def lib() -> C.CDLL:
     L.btdf_profile_read.argtypes = [ctxp, C.POINTER(C.c_double), C.POINTER(C.c_double),
                                     C.POINTER(C.c_int64), C.POINTER(C.c_int64)]
     L.btdf_tune.argtypes = [ctxp, C.c_int32, C.c_int32]
+    L.btdf_tune_pairs.argtypes = [ctxp, C.c_int32]
     L.btdf_device_bytes.argtypes = [ctxp, C.POINTER(C.c_size_t)]
     L.btdf_last_error.argtypes = [ctxp]
     L.btdf_last_error.restype = C.c_char_p
@@ -124,6 +125,7 @@ def lib() -> C.CDLL:
     L.btdf_batch_body_count.argtypes = [vp, C.POINTER(C.c_int32)]
     L.btdf_batch_body_lattice.argtypes = [vp, C.c_int32, C.POINTER(C.c_int32)]
     L.btdf_batch_tune.argtypes = [vp, C.c_int32]
+    L.btdf_batch_tune_pairs.argtypes = [vp, C.c_int32]
     L.btdf_batch_step.argtypes = [vp, C.c_int64]
     L.btdf_batch_sync.argtypes = [vp]
     L.btdf_batch_step_count.argtypes = [vp]
@@ -352,6 +354,10 @@ class Lattice:
         and an optional cap on its grid (0: the variant's default)."""
         self._check(lib().btdf_tune(self._ctx, int(variant), int(grid_blocks)), "btdf_tune")
 
+    def tune_pairs(self, on=True):
+        """Steps in pairs, or not, beside the variant of tune() (btdf_tune_pairs)."""
+        self._check(lib().btdf_tune_pairs(self._ctx, 1 if on else 0), "btdf_tune_pairs")
+
     def device_bytes(self) -> int:
         n = C.c_size_t()
         self._check(lib().btdf_device_bytes(self._ctx, C.byref(n)), "btdf_device_bytes")
@@ -478,6 +484,10 @@ class Batch:
 
     def tune(self, variant):
         self._check(lib().btdf_batch_tune(self._b, int(variant)), "btdf_batch_tune")
+
+    def tune_pairs(self, on=True):
+        """As Lattice.tune_pairs."""
+        self._check(lib().btdf_batch_tune_pairs(self._b, 1 if on else 0), "btdf_batch_tune_pairs")
 
     def autotune(self, steps=10, flush_l2=False):
         """Times launch shapes 1..4 on the batch (btdf_batch_autotune)."""

@@ -220,7 +220,7 @@ struct btdf_ctx {
     long long pf_units[2][2] = {};                 // L2 prefetch distance of variants 10, 11 [local/pull]
     long long tma_grid[kVarCount] = {};  // persistent grid of each TMA variant
     int variant = kVarAuto;              // LBM kernel variant (btdf_tune)
-    bool pairs_tuned = false;            // the autotuner found pairs of steps faster than `variant`
+    int pairs_mode = kPairsRule;
     int grid_override = 0;               // 0: SMs x resident blocks
     bool tma_ok = false;                 // tensor maps encoded
     CUtensorMap tmap[2][3];              // [buffer][box of 10 / 18 / 9 rows]
@@ -520,11 +520,10 @@ bool pairs_possible(const btdf_ctx* ctx) {
 // singly -> in pairs, with one body and the 3-point delta: 160 x 80 FP32 6.1 -> 4.7,
 // FP16 8.7 -> 5.3; 800 x 400 7.2 -> 5.7 and 8.4 -> 5.4; 1600 x 800 14.8 -> 11.5 and
 // 13.3 -> 10.7; with the 4-point cosine 160 x 80 6.1 -> 6.0 and 8.8 -> 6.4, 800 x 400
-// 7.2 -> 6.6 and 8.4 -> 6.7; 160 x 80 without bodies 3.7 -> 2.1), or after the autotuner
-// found them so.
+// 7.2 -> 6.6 and 8.4 -> 6.7; 160 x 80 without bodies 3.7 -> 2.1), or as was asked for.
 bool pairs_allowed(const btdf_ctx* ctx) {
     if (!pairs_possible(ctx)) return false;
-    if (ctx->variant != kVarAuto || ctx->grid_override != 0) return ctx->pairs_tuned;
+    if (ctx->pairs_mode != kPairsRule) return ctx->pairs_mode == kPairsOn;
     const int v = auto_variant(ctx), nx = ctx->cfg.nx;
     const int bcx = ctx->cfg.bc_x == BTDF_BCX_CONVECTIVE ? kBcxInout : ctx->cfg.bc_x;
     const int npl = pair_npl(ctx->cfg.storage, bcx, nx, ctx->cfg.ny);
@@ -1052,7 +1051,7 @@ int copy_history(btdf_ctx* ctx, int32_t body, int64_t first, int64_t n, double2*
 
 extern "C" {
 
-int btdf_version(void) { return 1; }
+int btdf_version(void) { return 2; }
 
 const char* btdf_status_string(int s) {
     switch (s) {
@@ -1570,8 +1569,14 @@ int btdf_tune(btdf_ctx* ctx, int32_t variant, int32_t grid_blocks) {
     CK(cudaStreamSynchronize(ctx->stream));
     drop_graphs(ctx);
     ctx->variant = variant;
-    ctx->pairs_tuned = false;
+    ctx->pairs_mode = variant == kVarAuto && grid_blocks == 0 ? kPairsRule : kPairsOff;
     ctx->grid_override = grid_blocks;
+    return BTDF_OK;
+}
+
+int btdf_tune_pairs(btdf_ctx* ctx, int32_t on) {
+    if (!ctx) return BTDF_EINVAL;
+    ctx->pairs_mode = on ? kPairsOn : kPairsOff;
     return BTDF_OK;
 }
 
@@ -1816,7 +1821,7 @@ int btdf_autotune(btdf_ctx* ctx, int32_t steps, int32_t flush_l2, int32_t* chose
     // restore the state, the counter and the last step's marker results
     ctx->tune_hist = nullptr;
     ctx->variant = rc == BTDF_OK ? best : var0;
-    if (rc == BTDF_OK) ctx->pairs_tuned = res[0] > 0.0f && res[0] < res[best];
+    if (rc == BTDF_OK) ctx->pairs_mode = res[0] > 0.0f && res[0] < res[best] ? kPairsOn : kPairsOff;
     ctx->cur = cur0;
     ctx->poststream = post0;
     ctx->steps = steps0;

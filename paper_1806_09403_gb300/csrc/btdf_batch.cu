@@ -85,7 +85,7 @@ struct btdf_batch {
     PairForces pf{};
     PairBatch pb{};
     bool gexec_pairs[2] = {false, false};
-    bool variant_set = false;              // btdf_batch_tune / autotune chose a launch shape
+    int pairs_mode = kPairsRule;
     double2* tune_hist = nullptr;          // one-slot force ring while btdf_batch_autotune times steps
 };
 
@@ -452,8 +452,11 @@ int64_t pair_worth(const btdf_batch* bt) {
     return (int64_t)((10.0 + 0.23 * m) / (6.0 + (bt->storage == kStoreF32 ? 3.2e-6 : 2.2e-6) * n + 2e-3 * m));
 }
 
-// Pairs of steps unless a launch shape was chosen: with every support inside.
-bool pairs_allowed(const btdf_batch* bt) { return !bt->variant_set && (bt->nmark == 0 || bt->markers_inside); }
+// Pairs of steps unless a launch shape was chosen without them: with every support
+// inside.  (Here they were the faster form at every size and width measured.)
+bool pairs_allowed(const btdf_batch* bt) {
+    return bt->pairs_mode != kPairsOff && (bt->nmark == 0 || bt->markers_inside);
+}
 
 BatchLbm lbm_params(const btdf_batch* bt, int s) {
     BatchLbm b{};
@@ -755,7 +758,13 @@ int btdf_batch_tune(btdf_batch* bt, int32_t variant) {
     BCK(cudaStreamSynchronize(bt->stream));
     drop_graphs(bt);
     bt->variant = variant == 0 ? 3 : variant;
-    bt->variant_set = variant != 0;
+    bt->pairs_mode = variant == 0 ? kPairsRule : kPairsOff;
+    return BTDF_OK;
+}
+
+int btdf_batch_tune_pairs(btdf_batch* bt, int32_t on) {
+    if (!bt) return BTDF_EINVAL;
+    bt->pairs_mode = on ? kPairsOn : kPairsOff;
     return BTDF_OK;
 }
 
@@ -840,7 +849,7 @@ int btdf_batch_autotune(btdf_batch* bt, int32_t steps, int32_t flush_l2, int32_t
     const int rc = run();
     bt->tune_hist = nullptr;
     bt->variant = rc == BTDF_OK ? best : var0;
-    if (rc == BTDF_OK) bt->variant_set = !(res[0] > 0.0f && res[0] < res[best]);
+    if (rc == BTDF_OK) bt->pairs_mode = res[0] > 0.0f && res[0] < res[best] ? kPairsOn : kPairsOff;
     bt->cur = cur0;
     bt->poststream = post0;
     cudaError_t e = cudaSuccess;

@@ -254,6 +254,9 @@ inline int single_columns(int nxp, int npl) { return (nxp + 32 * npl - 1) / (32 
 inline bool pair_needs_4(int bcx, int nx) { return bcx == kBcxInout && (nx - 1) % pair_own(2) == 0; }
 // Nodes per lane of the pair kernel for a lattice.
 int pair_npl(int storage, int bcx, int nx, int ny);
+// Whether steps go in pairs where they can: by the rules for variant 0, always, never
+// (btdf_tune, btdf_tune_pairs, the autotuners).
+enum : int { kPairsRule = 0, kPairsOn = 1, kPairsOff = 2 };
 // Whether pairs pay for `nodes` nodes that take them `pair` columns and single steps
 // `single` columns a row.
 bool pairs_pay(int storage, bool bodies, double nodes, double pair, double single);

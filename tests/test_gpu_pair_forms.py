@@ -170,3 +170,37 @@ def test_any_batch(seed):
         for body in range(len(a.bodies)):
             fa, fb = (x.forces(body, x.steps - k, k) for x in (a, b))
             assert np.array_equal(fa[0], fb[0]) and np.array_equal(fa[1], fb[1])
+
+
+def test_pairs_beside_a_chosen_variant():
+    """tune_pairs keeps the variant for the single steps that remain; tune undoes it."""
+    body = W.circle_markers(60.3, 30.2, 9.0, 28)
+    a, b = lattices(150, 61, B.BTDF_F32, W.BCX_INOUT, W.BCY_FREESLIP, [body])
+    a.tune(8)
+    before = a.device_bytes()
+    a.step(70)
+    assert a.device_bytes() == before
+    a.tune_pairs()
+    a.step(71)
+    assert a.device_bytes() > before   # the tables of pairs
+    b.step(141)
+    same(a, b, 8)
+    a.tune(2)
+    a.step(5)
+    a.tune_pairs(False)
+    a.step(2)
+    b.step(7)
+    same(a, b, 2)
+
+
+def test_batch_pairs_beside_a_chosen_shape():
+    cases = [W.small_cylinder(delta=3), W.small_cylinder(delta=3, seed=9)]
+    a, b = (B.Batch.from_cases(cases, history_len=64) for _ in range(2))
+    a.tune(2)
+    a.tune_pairs()
+    b.tune(1)
+    for n in (67, 40):
+        a.step(n)
+        b.step(n)
+        for i in range(2):
+            assert np.array_equal(a.field(i, B.FIELD_POPS), b.field(i, B.FIELD_POPS))
