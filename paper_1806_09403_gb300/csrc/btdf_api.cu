@@ -196,7 +196,6 @@ struct btdf_ctx {
     // [9][ny] outlet column of the last step (convective outlet): d_outlet[b]
     // belongs to population buffer b
     float* d_outlet[2] = {nullptr, nullptr};
-    int sms = 1;
     float2* d_box = nullptr;           // perimeter velocities of the prescribed-velocity box
     std::vector<MarkerAux> aux_host;
     // Pinned host staging, so per-step host <-> device copies are true DMA
@@ -815,9 +814,10 @@ int rebuild_markers(btdf_ctx* ctx) {
 size_t outlet_bytes(const btdf_ctx* ctx) { return ctx->d_outlet[0] ? sizeof(float) * 9 * ctx->cfg.ny : 0; }
 
 // Marker positions must be finite and their support must touch the lattice.
-// Under the convective outlet no support may reach the outlet column: the IB
-// kernel would read the outlet column buffer while the overlapping LBM kernel
-// rewrites it.  Every path that places markers (add, move) goes through here.
+// Under the convective outlet no support may reach the outlet column, whose
+// velocity is the boundary rule's and not the flow's to correct.  (The kernels
+// could read it: they take the column from one buffer and write it to the other.)
+// Every path that places markers (add, move) goes through here.
 int check_positions(btdf_ctx* ctx, int n, const double* X, const double* Y) {
     const int nx = ctx->cfg.nx, ny = ctx->cfg.ny;
     const double half = 0.5 * ctx->width;
@@ -1123,7 +1123,6 @@ int btdf_create(const btdf_config* cfg, void* stream, btdf_ctx** out) {
         if (cudaGetDevice(&dev) != cudaSuccess ||
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
             return bail(BTDF_ECUDA);
-        ctx->sms = sms;
         for (int v = 0; v < kVarCount; v++)
             if (is_tma(v)) ctx->tma_grid[v] = (long long)sms * collide_stream_tma_blocks_per_sm(c.storage, v);
         ctx->pf_grid[0] = (long long)sms * collide_stream_blocks_per_sm(c.storage, true, kVarReg4Pf);

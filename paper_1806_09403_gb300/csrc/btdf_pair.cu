@@ -161,8 +161,9 @@ __device__ __forceinline__ void collide_pairs(P2 (&f)[9][NP], const LatticeParam
 }
 
 // NPL neighbouring populations of one direction, as stored: packed FP32 pairs, or
-// 16-bit pairs.
+// 16-bit pairs (four of them: pair_npl).
 template <typename T, int NPL> struct Vec {
+    static_assert(NPL == 4, "16-bit storage takes 4 nodes per lane");
     static constexpr int NP = NPL / 2;
     unsigned w[NP];
     static __device__ __forceinline__ float2 to2(unsigned v) {
@@ -170,26 +171,17 @@ template <typename T, int NPL> struct Vec {
         else return Io16<__nv_bfloat16, __nv_bfloat162>::to2(v);
     }
     __device__ __forceinline__ void load(const T* p) {
-        if constexpr (NPL == 4) {
-            const uint2 v = __ldg(reinterpret_cast<const uint2*>(p));
-            w[0] = v.x;
-            w[1] = v.y;
-        } else {
-            w[0] = __ldg(reinterpret_cast<const unsigned*>(p));
-        }
+        const uint2 v = __ldg(reinterpret_cast<const uint2*>(p));
+        w[0] = v.x;
+        w[1] = v.y;
     }
     __device__ __forceinline__ void loads(const T* p) {   // shared memory
-        if constexpr (NPL == 4) {
-            const uint2 v = *reinterpret_cast<const uint2*>(p);
-            w[0] = v.x;
-            w[1] = v.y;
-        } else {
-            w[0] = *reinterpret_cast<const unsigned*>(p);
-        }
+        const uint2 v = *reinterpret_cast<const uint2*>(p);
+        w[0] = v.x;
+        w[1] = v.y;
     }
     __device__ __forceinline__ void store(T* p) const {
-        if constexpr (NPL == 4) *reinterpret_cast<uint2*>(p) = make_uint2(w[0], w[1]);
-        else *reinterpret_cast<unsigned*>(p) = w[0];
+        *reinterpret_cast<uint2*>(p) = make_uint2(w[0], w[1]);
     }
     __device__ __forceinline__ P2 get(int j) const {
         const float2 f = to2(w[j]);
@@ -860,7 +852,8 @@ namespace {
 
 template <typename T>
 cudaError_t pair_t(const void* gin, void* gout, const LatticeParams& p, const PairForces& q, bool pdl, cudaStream_t st) {
-    if (q.npl == 2) return pair_tn<T, 2, 8, 6, 5>(gin, gout, p, q, pdl, st);
+    if constexpr (sizeof(T) == 4)
+        if (q.npl == 2) return pair_tn<T, 2, 8, 6, 5>(gin, gout, p, q, pdl, st);
     return pair_tn<T, 4, 9, 7, 3>(gin, gout, p, q, pdl, st);
 }
 
@@ -881,7 +874,8 @@ cudaError_t pair_batch_tn(const void* gin, void* gout, const PairBatch& b, const
 template <typename T>
 cudaError_t pair_batch_t(const void* gin, void* gout, const PairBatch& b, const PairForces& q, bool pdl,
                          cudaStream_t st) {
-    if (q.npl == 2) return pair_batch_tn<T, 2, 8, 6, 5>(gin, gout, b, q, pdl, st);
+    if constexpr (sizeof(T) == 4)
+        if (q.npl == 2) return pair_batch_tn<T, 2, 8, 6, 5>(gin, gout, b, q, pdl, st);
     return pair_batch_tn<T, 4, 9, 7, 3>(gin, gout, b, q, pdl, st);
 }
 
