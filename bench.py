@@ -71,13 +71,16 @@ def measured_peaks():
         return None
 
 
+# The code that the single-step kernels are compiled from.
+KERNEL_SOURCES = ("btdf_kernels.cu", "btdf_device.cuh", "btdf_collide.cuh")
+
+
 def kernel_source_hash():
     """First 16 hex digits of the SHA-256 of the forward kernels' code
-    (btdf_kernels.cu followed by btdf_device.cuh) with comments removed and
-    whitespace collapsed, so that only a change of the code itself
-    invalidates a profile taken on it."""
+    (KERNEL_SOURCES in order) with comments removed and whitespace collapsed,
+    so that only a change of the code itself invalidates a profile taken on it."""
     h = hashlib.sha256()
-    for f in ("btdf_kernels.cu", "btdf_device.cuh"):
+    for f in KERNEL_SOURCES:
         src = open(os.path.join(ROOT, "paper_1806_09403_gb300", "csrc", f)).read()
         src = re.sub(r"/\*.*?\*/", " ", src, flags=re.S)
         src = re.sub(r"//[^\n]*", " ", src)
