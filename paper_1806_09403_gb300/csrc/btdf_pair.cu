@@ -7,9 +7,9 @@
 // second step needs the first step's result on its eight neighbours only.
 // pair_kernel keeps that result in shared memory, so a pair of steps moves what a
 // single one moves.  Measured, us a step, single -> pair: 8192 x 4096 with 400
-// bodies FP32 343 -> 232, FP16 220 -> 209; 1600 x 800 with one body FP32
-// 14.8 -> 11.6, FP16 13.3 -> 11.1; 1601 x 1601 BF16 28.2 -> 21.7; 128 lattices in
-// a batch FP32 395 -> 242.
+// bodies FP32 343 -> 231, FP16 220 -> 209; 1600 x 800 with one body FP32
+// 14.8 -> 11.5, FP16 13.3 -> 10.7; 1601 x 1601 BF16 with the convective outlet
+// 28.2 -> 20.5; 128 lattices in a batch FP32 395 -> 239.
 //
 // The marker forces of the second step are needed before the pass that would
 // produce the state they are interpolated from.  ib_pair_kernel redoes the
@@ -24,7 +24,9 @@
 // pair kernel off the band wait for none of them.  What is on the chain's path is
 // kept short: the kernels after ib_force have loaded everything but the forces
 // (state, tables, the first terms of every spread) before they wait.  With those
-// loads after the wait, entry by entry, a pair on 160 x 80 took 12.7 us, now 9.8.
+// loads after the wait, entry by entry, a pair on 160 x 80 with the 3-point delta took
+// 12.7 us, now 9.4; with the 4-point cosine, whose 36 patch nodes take a warp two
+// rounds, it takes 11.9 (two single steps 12.2).
 #include "btdf_internal.cuh"
 #include "btdf_device.cuh"
 #include "btdf_collide.cuh"
@@ -277,11 +279,14 @@ template <int NPL> struct Vec<float, NPL> {
 // warp takes a row at a time, NPL consecutive nodes per lane; the outer two lanes
 // hold the columns beside the tile.
 //
-// What bounds it: instructions.  On 8192 x 4096 FP32 it moves 2.42 GB a pair at
-// 5.2 TB/s (0.78 of the measured copy rate), FP16 half the bytes in nearly the same
-// time; on 4096 x 2048 the issue slots are 65% (FP32) and 72% (FP16) busy, with the
-// FMA pipe throttling; FP32 arithmetic is 77 of about 300 instructions per row of
-// 64 nodes and step.  Small tiles, although their halo costs 14-20% more node
+// What bounds it: instructions, FP32 nearly as much the traffic.  On 8192 x 4096 FP32
+// it moves 2.42 GB a pair at 5.2 TB/s (0.78 of the measured copy rate), FP16 half the
+// bytes in nearly the same time; under ncu on 4096 x 2048 the issue slots are 52%
+// (FP32) and 62% (FP16) busy and DRAM 62% and 32%, with 273 and 297 warp instructions
+// per 64 nodes and step, halo included.  The register caps cost spills, of boundary
+// code for the most part: 164 bytes a thread in FP32 with 4 nodes per lane, 64 with 2,
+// 24 in FP16, 156 in BF16; in the batch, whose constants come from shared memory, 448,
+// 164, 236 and 444.  Small tiles, although their halo costs 14-20% more node
 // updates, keep the register count low and 3 to 5 blocks an SM resident, so that one block's
 // barrier and loads hide behind the others: tiles of 14 rows with two blocks an SM
 // took 235 to 265 us a step on 8192 x 4096.
@@ -818,13 +823,13 @@ cudaError_t ib_pair_t(int width, const void* g, const LatticeParams& p, const Ib
 }  // namespace
 
 // Nodes per lane.  FP32 below 2^22 nodes: 2, with 40 warps an SM in tiles of 60 x 6
-// (11.6 us a step at 1600 x 800 against 12.2 with 4); above, where fewer
+// (11.5 us a step at 1600 x 800 against 12.2 with 4); above, where fewer
 // instructions per node count for more, 4, with 27 warps in tiles of 120 x 7
 // (232 us at 8192 x 4096 against 243), unless its strips leave many columns unused
-// (128 x 65536: 139 us with 4, 105 with 2, 110 singly). 
-// 16-bit storage: 4 (1600 x 800 11.1 against 11.4, 8192 x 4096 209 against 239).  Also measured with 4: tiles of 120 x 6 with
-// four blocks an SM (FP32 234, FP16 207 at 8192 x 4096, 11.3 at 1600 x 800), 120 x 8
-// with three (240, 209, 11.4).
+// (128 x 65536: 139 us with 4, 105 with 2, 110 singly).  16-bit storage: 4 (2 took
+// 11.4 us at 1600 x 800, now 10.7, and 239 at 8192 x 4096 against 209).  Also measured
+// with 4: tiles of 120 x 6 with four blocks an SM (FP32 234, FP16 207 at 8192 x 4096,
+// 11.3 at 1600 x 800), 120 x 8 with three (240, 209, 11.4).
 int pair_npl(int storage, int bcx, int nx, int ny) {
     if (storage != kStoreF32 || pair_needs_4(bcx, nx)) return 4;
     return (long long)nx * ny >= (1ll << 22) && pair_wide(pair_columns(nx, 2), pair_columns(nx, 4)) ? 4 : 2;
