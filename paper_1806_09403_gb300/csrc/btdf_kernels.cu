@@ -1034,8 +1034,8 @@ __global__ void init_kernel(T* g, LatticeParams p, const double* rho, const doub
 // out together (gather_node); through read_node's out-of-line pull with its
 // stack array the populations of 8192 x 4096 took 884 us to read in FP32; the pass
 // that steps 50 times and reads them went from 12.66 to 12.11 ms.  With blocks for
-// every row, reading 2^22 nodes 4 wide took 1472 us (FP16 1567), now 225 (139); 64
-// wide 157 (188), now 85 (81).
+// every row, reading 2^22 nodes 4 wide took 1472 us (FP16 1567), now 235 (146); 64
+// wide 157 (188), now 83 (83).
 // kFold: the populations of inlet and outlet nodes come from the node beside them,
 // so its loads go out with the rest of the warp's and the rule follows; on its own
 // path the row ends' loads double a narrow lattice's time (64 wide 136 us).
